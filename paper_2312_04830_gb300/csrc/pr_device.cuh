@@ -68,10 +68,11 @@ struct SpeciesRec {
 // ------------------------------------------------------------------ math
 template <typename T> struct M;
 template <> struct M<double> {
-    static __device__ __forceinline__ double sqrt(double x) { return ::sqrt(x); }
-    static __device__ __forceinline__ double rsqrt(double x) { return ::rsqrt(x); }
-    static __device__ __forceinline__ double cbrt(double x) { return ::cbrt(x); }
-    // table-driven forms with fewer FP64-pipe operations (pr_math64.cuh)
+    // forms on the integer pipe (pr_math64.cuh)
+    static __device__ __forceinline__ double rcp(double x) { return m64::rcp(x); }
+    static __device__ __forceinline__ double div(double a, double b) { return m64::div(a, b); }
+    static __device__ __forceinline__ double sqrt(double x) { return m64::sqrt(x); }
+    static __device__ __forceinline__ double cbrt(double x) { return m64::cbrt(x); }
     static __device__ __forceinline__ double log(double x) { return m64::log(x); }
     static __device__ __forceinline__ double log1p(double x) { return m64::log1p(x); }
     static __device__ __forceinline__ double exp(double x) { return m64::exp(x); }
@@ -83,8 +84,9 @@ template <> struct M<double> {
     static constexpr double eps = 2.220446049250313e-16;
 };
 template <> struct M<float> {
+    static __device__ __forceinline__ float rcp(float x) { return 1.f / x; }
+    static __device__ __forceinline__ float div(float a, float b) { return a / b; }
     static __device__ __forceinline__ float sqrt(float x) { return ::sqrtf(x); }
-    static __device__ __forceinline__ float rsqrt(float x) { return ::rsqrtf(x); }
     static __device__ __forceinline__ float cbrt(float x) { return ::cbrtf(x); }
     static __device__ __forceinline__ float log(float x) { return ::logf(x); }
     static __device__ __forceinline__ float log1p(float x) { return ::log1pf(x); }
@@ -96,6 +98,46 @@ template <> struct M<float> {
     static __device__ __forceinline__ float nan() { return __int_as_float(0x7fc00000); }
     static constexpr float eps = 1.1920929e-07f;
 };
+
+// 1/a and 1/b, and a/b and b/a.  In FP32 the pair shares one division; in
+// FP64 each takes its own, the products of the shared form being FP64-pipe
+// operations and the integer-pipe divisions not (rcp ~13 cycles of issue per
+// warp and SM, a DMUL 16).
+template <typename Real>
+__device__ __forceinline__ void inv_pair(Real a, Real b, Real &ia, Real &ib)
+{
+    if constexpr (sizeof(Real) == 8) {
+        ia = M<Real>::rcp(a);
+        ib = M<Real>::rcp(b);
+    } else {
+        const Real r = Real(1) / (a * b);
+        ia = b * r;
+        ib = a * r;
+    }
+}
+
+template <typename Real>
+__device__ __forceinline__ void quot_pair(Real a, Real b, Real &q, Real &iq)
+{
+    if constexpr (sizeof(Real) == 8) {
+        q = M<Real>::div(a, b);
+        iq = M<Real>::div(b, a);
+    } else {
+        const Real r = Real(1) / (a * b);
+        q = a * a * r;
+        iq = b * b * r;
+    }
+}
+
+// x^-b for x > 0 and a constant b in (0, 1)
+template <typename Real>
+__device__ __forceinline__ Real pow_neg(Real x, double b)
+{
+    if constexpr (sizeof(Real) == 8)
+        return m64::pow_neg(x, (uint64_t)(b * 18446744073709551616.0));
+    else
+        return M<Real>::exp(Real(-b) * M<Real>::log(x));
+}
 
 // -------------------------------------------------------- composition
 // T-independent part of a cell: mole fractions, mean molar mass, b_m.
@@ -159,7 +201,7 @@ __device__ __forceinline__ bool load_comp(Comp<Real, NS> &c, const Real *__restr
         s += c.x[k];
     }
     ok = ok && (M<Real>::fabs(ysum - Real(1)) <= Real(1e-6)) && (s > Real(0));
-    Real inv_s = Real(1) / s;
+    Real inv_s = M<Real>::rcp(s);
     Real bm = 0;
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
@@ -178,9 +220,9 @@ __device__ __forceinline__ void mix_a(const Comp<Real, NS> &c, Real T, const Spe
                                       const Real *kij1m, Real &am, Real &dam, Real &d2am)
 {
     const Real sqT = M<Real>::sqrt(T);
-    const Real isqT = Real(1) / sqT;
+    const Real isqT = M<Real>::rcp(sqT);
     const Real h1 = Real(-0.5) * isqT;          // d sqrt(T)/dT factor (with sign)
-    const Real h2 = Real(0.25) * isqT / T;
+    const Real h2 = M<Real>::div(Real(0.25) * isqT, T);
     if (!KIJ) {
         Real S0 = 0, S1 = 0, S2 = 0;
 #pragma unroll
@@ -238,7 +280,7 @@ __device__ __forceinline__ RZ cubic_polish(RZ z, RZ c2, RZ c1, RZ c0)
         const RZ f = M<RZ>::fma(M<RZ>::fma(z + c2, z, c1), z, c0);
         const RZ d = M<RZ>::fma(M<RZ>::fma(RZ(3), z, RZ(2) * c2), z, c1);
         if (d == RZ(0)) break;
-        const RZ dz = f / d;
+        const RZ dz = M<RZ>::div(f, d);
         z -= dz;
         if (M<RZ>::fabs(dz) <= RZ(2) * M<RZ>::eps * M<RZ>::fabs(z)) break;
     }
@@ -315,7 +357,8 @@ template <typename RZ>
 __device__ __forceinline__ RZ pr_gres(RZ Z, RZ A, RZ B)
 {
     const RZ dp = RZ(1.0 + kSqrt2), dm = RZ(1.0 - kSqrt2);
-    return Z - RZ(1) - M<RZ>::log(Z - B) - A / (RZ(2.0 * kSqrt2) * B) * M<RZ>::log((Z + dp * B) / (Z + dm * B));
+    return Z - RZ(1) - M<RZ>::log(Z - B) -
+           M<RZ>::div(A, RZ(2.0 * kSqrt2) * B) * M<RZ>::log(M<RZ>::div(Z + dp * B, Z + dm * B));
 }
 
 // Select the physical root: the one of least residual Gibbs energy; ties
@@ -410,9 +453,7 @@ __device__ __forceinline__ void thermo(const Comp<Real, NS> &c, Real T, Real p, 
         }
     }
     if (need_rz) {
-        // pairs of quotients below share one reciprocal (an FP64 division is
-        // several FP64-pipe instructions)
-        const RZ iRT = RZ(1) / (RZ)RT;
+        const RZ iRT = M<RZ>::rcp((RZ)RT);
         const RZ pRT = (RZ)p * iRT;
         const RZ B = (RZ)bm * pRT;
         const RZ A = (RZ)am * pRT * iRT;
@@ -424,7 +465,7 @@ __device__ __forceinline__ void thermo(const Comp<Real, NS> &c, Real T, Real p, 
         o.nroots = nr;
         o.status = select_root<RZ>(zr, nr, A, B, Zz);
         if (o.status == kNoRoot) return;
-        larg = RZ(2.0 * kSqrt2) * B / (Zz + RZ(1.0 - kSqrt2) * B);
+        larg = M<RZ>::div(RZ(2.0 * kSqrt2) * B, Zz + RZ(1.0 - kSqrt2) * B);
     }
 
     // ideal-gas part (NASA-7), molar
@@ -450,9 +491,15 @@ __device__ __forceinline__ void thermo(const Comp<Real, NS> &c, Real T, Real p, 
             h_ig = M<Real>::fma(c.x[k], hk, h_ig);
         }
     }
-    const Real rWb = Real(1) / (c.Wbar * bm);
-    const Real iW = bm * rWb;                                         // 1 / Wbar
-    const Real inv2s2b = Real(1.0 / (2.0 * kSqrt2)) * c.Wbar * rWb;   // 1 / (2 sqrt 2 bm)
+    Real iW, inv2s2b;   // 1 / Wbar, 1 / (2 sqrt 2 bm)
+    if constexpr (sizeof(Real) == 8) {
+        iW = M<Real>::rcp(c.Wbar);
+        inv2s2b = M<Real>::rcp(Real(2.0 * kSqrt2) * bm);
+    } else {
+        const Real rWb = Real(1) / (c.Wbar * bm);
+        iW = bm * rWb;
+        inv2s2b = Real(1.0 / (2.0 * kSqrt2)) * c.Wbar * rWb;
+    }
 
     // departures (in RZ where the root enters, then Real)
     // ln[(Z + (1 + sqrt 2) B)/(Z + (1 - sqrt 2) B)] = log1p(2 sqrt 2 B / (Z + (1 - sqrt 2) B)):
@@ -473,16 +520,15 @@ __device__ __forceinline__ void thermo(const Comp<Real, NS> &c, Real T, Real p, 
     }
     const Real cv_dep = T * d2am * inv2s2b * Lr;
     const Real ZRT = Z * RT;
-    const Real rzp = Real(1) / (ZRT * p);
-    const Real V = ZRT * ZRT * rzp;                                   // Z R T / p
-    const Real rho_mol = p * p * rzp;                                 // p / (Z R T)
+    Real V, rho_mol;   // Z R T / p and its inverse
+    quot_pair<Real>(ZRT, p, V, rho_mol);
     const Real Vmb = V - bm;
     const Real den = M<Real>::fma(V, V + Real(2) * bm, -bm * bm);
-    const Real rvd = Real(1) / (Vmb * den);
-    const Real iVmb = den * rvd, iden = Vmb * rvd;
+    Real iVmb, iden;
+    inv_pair<Real>(Vmb, den, iVmb, iden);
     const Real dpdT = Real(kR) * iVmb - dam * iden;
     const Real dpdV = -RT * iVmb * iVmb + Real(2) * am * (V + bm) * iden * iden;
-    const Real cp_dep = cv_dep - T * dpdT * dpdT / dpdV - Real(kR);
+    const Real cp_dep = cv_dep - M<Real>::div(T * dpdT * dpdT, dpdV) - Real(kR);
     o.Z = Z;
     o.rho_mol = rho_mol;
     o.h = (h_ig + h_dep) * iW;
@@ -553,35 +599,44 @@ template <typename Real>
 __device__ __forceinline__ void chung_dense(Real Tc, Real Vc, Real cVc, Real omega, Real Mg, Real mur4, Real kap,
                                             Real T, Real rho_mol, Real cv_molar, Real &mu, Real &lam)
 {
-    // pairs of quotients share one reciprocal (FP64 divisions are costly)
-    const Real rTM = Real(1) / (Tc * Mg);
-    const Real Tr = T * Mg * rTM;                  // T / Tc
-    const Real iMg = Tc * rTM;                     // 1 / M
+    Real Tr, iMg;   // T / Tc, 1 / M
+    if constexpr (sizeof(Real) == 8) {
+        Tr = M<Real>::div(T, Tc);
+        iMg = M<Real>::rcp(Mg);
+    } else {
+        const Real rTM = Real(1) / (Tc * Mg);
+        Tr = T * Mg * rTM;
+        iMg = Tc * rTM;
+    }
     const Real sTr = M<Real>::sqrt(Tr);
     const Real sMTc = M<Real>::sqrt(Mg * Tc);
     const Real Ts = Real(1.2593) * Tr;
     const Real Fc = Real(1) - Real(0.2756) * omega + Real(0.059035) * mur4 + kap;
-    const Real lnTs = M<Real>::log(Ts);
-    const Real Ov = Real(1.16145) * M<Real>::exp(Real(-0.14874) * lnTs) + Real(0.52487) * M<Real>::exp(Real(-0.77320) * Ts)
+    const Real Ov = Real(1.16145) * pow_neg<Real>(Ts, 0.14874) + Real(0.52487) * M<Real>::exp(Real(-0.77320) * Ts)
                     + Real(2.16178) * M<Real>::exp(Real(-2.43787) * Ts);
     const Real y = rho_mol * Real(1e-6) * Vc * Real(1.0 / 6.0);
     const Real omy = Real(1) - y;
     const Real omy3 = omy * omy * omy;
     const Real yp = (y > Real(0)) ? y : Real(1);   // y = 0 only for p = 0, kept finite
-    const Real ryo = Real(1) / (omy3 * yp);
-    const Real G1 = (Real(1) - Real(0.5) * y) * yp * ryo;   // (1 - y/2) / (1 - y)^3
+    Real G1, iy;   // (1 - y/2) / (1 - y)^3, 1 / y
+    if constexpr (sizeof(Real) == 8) {
+        G1 = M<Real>::div(Real(1) - Real(0.5) * y, omy3);
+        iy = M<Real>::rcp(yp);
+    } else {
+        const Real ryo = Real(1) / (omy3 * yp);
+        G1 = (Real(1) - Real(0.5) * y) * yp * ryo;
+        iy = omy3 * ryo;
+    }
     Real E[10];
 #pragma unroll
     for (int i = 0; i < 10; ++i)
         E[i] = chung_visc<Real>(i, 0) + chung_visc<Real>(i, 1) * omega + chung_visc<Real>(i, 2) * mur4 + chung_visc<Real>(i, 3) * kap;
-    const Real iy = omy3 * ryo;                    // 1 / y
     const Real fy4 = (y > Real(0)) ? -M<Real>::expm1(-E[3] * y) * iy : E[3];
     const Real nG = E[0] * fy4 + E[1] * G1 * M<Real>::exp(E[4] * y) + E[2] * G1;
     const Real dG = E[0] * E[3] + E[1] + E[2];
-    const Real rG = Real(1) / (nG * dG);
-    const Real G2 = nG * nG * rG, iG2 = dG * dG * rG;
-    const Real rTO = Real(1) / (Ts * Ov);
-    const Real iTs = Ov * rTO, iOv = Ts * rTO;
+    Real G2, iG2, iTs, iOv;
+    quot_pair<Real>(nG, dG, G2, iG2);
+    inv_pair<Real>(Ts, Ov, iTs, iOv);
     const Real etass = E[6] * y * y * G2 * M<Real>::exp(E[7] + iTs * (E[8] + E[9] * iTs));
     const Real sqTs = Real(1.1221853679316978) * sTr;   // sqrt(1.2593) sqrt(Tr)
     const Real etas = sqTs * iOv * Fc * (iG2 + E[5] * y) + etass;
@@ -590,8 +645,13 @@ __device__ __forceinline__ void chung_dense(Real Tc, Real Vc, Real cVc, Real ome
     const Real be = Real(0.7862) - Real(0.7109) * omega + Real(1.3168) * omega * omega;
     const Real Zp = Real(2.0) + Real(10.5) * Tr * Tr;
     const Real dPsi = Real(0.6366) + be * Zp + Real(1.061) * al * be;
-    const Real rPV = Real(1) / (dPsi * cVc2);
-    const Real iVc23 = dPsi * rPV;                 // Vc^(-2/3)
+    Real iVc23, rPV = Real(0);   // Vc^(-2/3); FP32: 1 / (dPsi Vc^(2/3)), shared with Psi below
+    if constexpr (sizeof(Real) == 8) {
+        iVc23 = M<Real>::rcp(cVc2);
+    } else {
+        rPV = Real(1) / (dPsi * cVc2);
+        iVc23 = dPsi * rPV;
+    }
     mu = etas * Real(36.344e-7) * sMTc * iVc23;
     const Real eta0 = Real(40.785e-7) * Fc * (sMTc * sTr) * iVc23 * iOv;   // sqrt(M T)
     Real Bc[7];
@@ -601,10 +661,13 @@ __device__ __forceinline__ void chung_dense(Real Tc, Real Vc, Real cVc, Real ome
     const Real fyb4 = (y > Real(0)) ? -M<Real>::expm1(-Bc[3] * y) * iy : Bc[3];
     const Real nH = Bc[0] * fyb4 + Bc[1] * G1 * M<Real>::exp(Bc[4] * y) + Bc[2] * G1;
     const Real dH = Bc[0] * Bc[3] + Bc[1] + Bc[2];
-    const Real rH = Real(1) / (nH * dH);
-    const Real H2 = nH * nH * rH, iH2 = dH * dH * rH;
-    const Real Psi = Real(1) + al * (Real(0.215) + Real(0.28288) * al - Real(1.061) * be + Real(0.26665) * Zp) *
-                                   cVc2 * rPV;
+    Real H2, iH2;
+    quot_pair<Real>(nH, dH, H2, iH2);
+    Real Psi;
+    if constexpr (sizeof(Real) == 8)
+        Psi = Real(1) + M<Real>::div(al * (Real(0.215) + Real(0.28288) * al - Real(1.061) * be + Real(0.26665) * Zp), dPsi);
+    else
+        Psi = Real(1) + al * (Real(0.215) + Real(0.28288) * al - Real(1.061) * be + Real(0.26665) * Zp) * cVc2 * rPV;
     const Real iMkg = Real(1e3) * iMg;
     const Real q = Real(3.586e-3) * (Real(31.622776601683793) * sMTc * iMg) * iVc23;   // sqrt(Tc / M[kg/mol])
     lam = Real(31.2) * eta0 * Psi * iMkg * (iH2 + Bc[5] * y) + q * Bc[6] * y * y * sTr * H2;
@@ -654,17 +717,17 @@ __device__ __forceinline__ void transport(const Comp<Real, NS> &c, Real T, const
         Q = M<Real>::fma(Real(2) * c.x[i], t, Q);
     }
     const Real s3 = P1 * P1;                      // sigma_m^3
-    const Real iP1 = Real(1) / P1;
+    const Real iP1 = M<Real>::rcp(P1);
     const Real em = P2 * P2 * iP1 * iP1;          // (eps/k)_m
     const Real wm = P3 * iP1;                     // omega_m
     const Real mu4 = s3 * P4 * P4;                // mu_m^4 [debye^4]
     const Real km = P5 * P5;                      // kappa_m
     const Real sm = M<Real>::cbrt(s3);
-    const Real sqM = Q / (em * sm * sm);
+    const Real sqM = M<Real>::div(Q, em * sm * sm);
     const Real Mm = sqM * sqM;
     const Real Vcm = s3 * Real(1.0 / (0.809 * 0.809 * 0.809));
     const Real Tcm = Real(1.2593) * em;
-    const Real murd = Real(131.3 * 131.3) / (Vcm * Tcm);   // mu_r^2 / mu^2
+    const Real murd = M<Real>::div(Real(131.3 * 131.3), Vcm * Tcm);   // mu_r^2 / mu^2
     const Real mur4 = mu4 * murd * murd;
     chung_dense<Real>(Tcm, Vcm, sm * Real(1.0 / 0.809), wm, Mm, mur4, km, T, th.rho_mol, th.cv_ig_molar, mu, lam);
 }
@@ -697,7 +760,7 @@ __device__ __forceinline__ void fallback_cell_fp64(int64_t i, const float *__res
         s += c.x[k];
     }
     ok = ok && fabs(ysum - 1.0) <= 1e-6 && s > 0;
-    const double is = 1.0 / s;
+    const double is = M<double>::rcp(s);
     double bm = 0;
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
@@ -715,7 +778,7 @@ __device__ __forceinline__ void fallback_cell_fp64(int64_t i, const float *__res
         if (th.status != kNoRoot) {
             double mu, lam;
             transport<double, NS>(c, Tv, th, sp, pair, flags, mu, lam);
-            o[0] = (float)(pv * c.Wbar / (th.Z * kR * Tv));
+            o[0] = (float)M<double>::div(pv * c.Wbar, th.Z * kR * Tv);
             o[1] = (float)th.Z;
             o[2] = (float)th.h;
             o[3] = (float)th.cp;

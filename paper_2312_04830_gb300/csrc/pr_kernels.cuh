@@ -104,13 +104,13 @@ struct PropsArgs {
 template <typename Real>
 __device__ __forceinline__ Real psi_h(const Thermo<Real> &th, Real T, Real W)
 {
-    const Real V = Real(1) / th.rho_mol;
+    const Real V = M<Real>::rcp(th.rho_mol);
     const Real iV2 = th.rho_mol * th.rho_mol;
-    const Real dV_dT = -th.dpdT / th.dpdV;
-    const Real drho_dp_T = -W * iV2 / th.dpdV;
+    const Real dV_dT = M<Real>::div(-th.dpdT, th.dpdV);
+    const Real drho_dp_T = M<Real>::div(-W * iV2, th.dpdV);
     const Real drho_dT_p = -W * iV2 * dV_dT;
     const Real dh_dp_T = V - T * dV_dT;
-    return drho_dp_T - drho_dT_p * dh_dp_T / (th.cp * W);
+    return drho_dp_T - M<Real>::div(drho_dT_p * dh_dp_T, th.cp * W);
 }
 
 // resident CTAs per SM the property kernels ask the compiler to allow for
@@ -158,14 +158,14 @@ __global__ void __launch_bounds__(kBlock, props_min_blocks<Real>()) props_kernel
         }
         const bool good = ok && th.status != kNoRoot;
         const Real nanv = M<Real>::nan();
-        if (a.rho) a.rho[i] = good ? p * c.Wbar / (th.Z * Real(kR) * T) : nanv;
+        if (a.rho) a.rho[i] = good ? M<Real>::div(p * c.Wbar, th.Z * Real(kR) * T) : nanv;
         if (a.Z) a.Z[i] = good ? th.Z : nanv;
         if (a.h) a.h[i] = good ? th.h : nanv;
         if (a.cp) a.cp[i] = good ? th.cp : nanv;
         if (a.mu) a.mu[i] = good ? mu : nanv;
         if (a.lam) a.lam[i] = good ? lam : nanv;
         if (a.psi) a.psi[i] = good ? psi_h<Real>(th, T, c.Wbar) : nanv;
-        if (a.alpha) a.alpha[i] = good ? lam / th.cp : nanv;
+        if (a.alpha) a.alpha[i] = good ? M<Real>::div(lam, th.cp) : nanv;
         if (a.status) a.status[i] = th.status;
     }
 }
@@ -351,7 +351,7 @@ __device__ __forceinline__ int newton_solve(const Comp<Real, NS> &c, double hs, 
         const double f = h - hs;
         if (fabs(f) <= rtol * fmax(fabs(hs), fabs(cp) * T)) { st = kOk; Tres = T; break; }
         if (f < 0) lo = T; else hi = T;
-        double Tn = T - f / cp;
+        double Tn = T - M<double>::div(f, cp);
         const bool newton_ok = (cp > 0) && (Tn > lo) && (Tn < hi) && (fabs(f) <= 0.5 * fabs(fprev));
         if (!newton_ok) Tn = 0.5 * (lo + hi);
         if (!newton_ok && ((lo == kTLo && !lo_done) || (hi == kTHi && !hi_done))) {
@@ -390,7 +390,7 @@ __device__ __forceinline__ double cp_ideal_mass(const Comp<Real, NS> &c, Real T,
         const Real cpk = M<Real>::fma(M<Real>::fma(M<Real>::fma(M<Real>::fma(a[4], T, a[3]), T, a[2]), T, a[1]), T, a[0]);
         s = M<Real>::fma(c.x[k], cpk, s);
     }
-    return (double)s / (double)c.Wbar;
+    return M<double>::div((double)s, (double)c.Wbar);
 }
 
 // Composition in FP64 from FP32 mass fractions (the FP64 re-solve of the
@@ -410,7 +410,7 @@ __device__ __forceinline__ bool comp_fp64_of_fp32(Comp<double, NS> &c, const flo
         s += c.x[k];
     }
     ok = ok && (fabs(ysum - 1.0) <= 1e-6) && (s > 0.0);
-    const double inv_s = 1.0 / s;
+    const double inv_s = M<double>::rcp(s);
     double bm = 0;
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
@@ -482,7 +482,7 @@ __device__ __forceinline__ void newton_fp64_queued(const NewtonArgs<double> &a, 
                     FirstEval f = eval_h_first<double, double, NS, KIJ>(c, T, p, s.sp, s.kij, a.tmid_u);
                     f.cp = (double)cp32;
                     if (f.status != kNoRoot) {
-                        const double dT = (f.cp > 0.0) ? -(f.h - hs) / f.cp : 0.0;
+                        const double dT = (f.cp > 0.0) ? M<double>::div(-(f.h - hs), f.cp) : 0.0;
                         if (one_step_ok<NS>(f, T, dT, c.Wbar, s32.sp, (float)a.tmid_u)) {
                             a.Tout[i] = T + dT;
                             a.status[i] = kOk;

@@ -1,56 +1,37 @@
-// FP64 exp, expm1, log and log1p for the FP64 property paths, written for
-// fewer FP64-pipe operations than general library calls: the FP64 pipe is
-// the scarce unit of these kernels (2 operations per clock per SM on GB300),
-// and the exponentials and logarithms of Chung's correlation and of the
-// departure functions take about a third of its slots.
-//
-// exp: Tang's table-driven method (P. T. P. Tang, "Table-driven
-// implementation of the exponential function in IEEE floating-point
-// arithmetic", ACM TOMS 15 (1989) 144-157) with 64 table points: x =
-// (64 m + j) ln2/64 + r, |r| <= ln2/128, exp(x) = 2^m 2^(j/64) e^r, the
-// reduction in double-double by FMA, e^r - 1 by its Taylor polynomial to r^5
-// (the next term is below 3.4e-17 of the result; to r^7 for expm1, whose
-// result can be of the size of r), 2^(j/64) as a double-double table, 2^m
-// added to the exponent field.  11 FP64 operations (expm1: 15).
-// log: Tang's table-driven logarithm (ACM TOMS 16 (1990) 378-400) with
-// F = 1 + j/128 nearest the significand m: ln x = e ln2 + ln F + ln(1 + r),
+// FP64 elementary functions of the property paths.  The FP64 pipe is their
+// scarce unit (2 operations per clock per SM on GB300), so the usual argument
+// ranges are computed on the integer pipe (pr_int64.cuh, at most 0.6 units in
+// the last place before any range restriction below); what they leave goes to
+// the forms here, or to CUDA's functions:
+//   rcp, div, sqrt   normal operands and results;
+//   exp              |x| < 64 (else CUDA's exp);
+//   expm1            2^-7 <= |x| < 64 (smaller: Tang's form below);
+//   log, log1p       where |ln| is at least 2^-5 (nearer zero: Tang's form);
+//   pow_neg, cbrt    x^-b for a constant b in (0, 1), x^(1/3), normal x > 0 (cbrt: x >= 0).
+// Tang's table-driven forms (P. T. P. Tang, ACM TOMS 15 (1989) 144-157 and 16
+// (1990) 378-400), with FP64 operations:
+// exp: 64 table points: x = (64 m + j) ln2/64 + r, |r| <= ln2/128, exp(x) =
+// 2^m 2^(j/64) e^r, the reduction in double-double by FMA, e^r - 1 by its
+// Taylor polynomial to r^7 (expm1, whose result can be of the size of r),
+// 2^(j/64) as a double-double table.
+// log: F = 1 + j/128 nearest the significand m: ln x = e ln2 + ln F + ln(1 + r),
 // r = (m - F)/F (m - F exact; 1/F from a table and one correction step),
-// ln(1 + r) by its Taylor polynomial to r^8 (|r| <= 1/256).  18 FP64
-// operations.
-// Valid for finite positive normal x; exp for |x| < 512 (larger |x|, NaN and
-// infinities go to CUDA's exp).  Errors on the tested ranges
-// (tests/test_gpu_math64.py, extended-precision references): exp 0.75 ulp,
-// expm1 1.44, log 1.00, log1p 1.46 at most (CUDA's: 0.85, 1.05, 0.50, 1.46).
+// ln(1 + r) by its Taylor polynomial to r^8 (|r| <= 1/256).
+// Errors on the tested ranges (tests/test_gpu_math64.py, extended-precision
+// references): within 1.5 ulp.
 #pragma once
 
 #include <cuda_runtime.h>
 
 #include "math64_tables.h"
+#include "pr_int64.cuh"
 
 namespace m64 {
 
 // round-to-nearest integer of x * 64/ln2 via the 1.5 * 2^52 shifter
 constexpr double kShift = 6755399441055744.0;
 
-// |x| < 512, from the exponent field of the high word (integer pipe)
-__device__ __forceinline__ bool exp_in_range(double x)
-{
-    return ((__double2hiint(x) >> 20) & 0x7FF) < 1023 + 9;
-}
-
-// e^r - 1 for |r| <= ln2/128, to the r^5 term: the truncation is below
-// 3.4e-17 of 1 + p, enough for exp
-__device__ __forceinline__ double expm1_small(double r)
-{
-    const double r2 = r * r;
-    double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
-    q = fma(q, r, 1.0 / 6.0);
-    q = fma(q, r, 0.5);
-    return fma(q, r2, r);
-}
-
-// the same to the r^7 term: the truncation is below 5e-18 of p itself, as
-// expm1 needs when its result is of the size of r
+// e^r - 1 for |r| <= ln2/128: the truncation is below 5e-18 of it
 __device__ __forceinline__ double expm1_small_rel(double r)
 {
     const double r2 = r * r;
@@ -62,26 +43,10 @@ __device__ __forceinline__ double expm1_small_rel(double r)
     return fma(q, r2, r);
 }
 
-__device__ __forceinline__ double exp(double x)
-{
-    if (!exp_in_range(x)) return ::exp(x);
-    const double t = fma(x, k64OverLn2, kShift);
-    const double kd = t - kShift;
-    const int k = __double2loint(t);
-    double r = fma(-kd, kLn2Over64Hi, x);
-    r = fma(-kd, kLn2Over64Lo, r);
-    const double p = expm1_small(r);
-    const int j = k & 63, m = k >> 6;
-    const double th = __ldg(&kExp2Hi[j]), tl = __ldg(&kExp2Lo[j]);
-    const double v = th + fma(th, p, tl);
-    return __hiloint2double(__double2hiint(v) + (m << 20), __double2loint(v));
-}
-
-// e^x - 1: as exp, with the 1 taken off before the scaled table value is
+// e^x - 1 for |x| < 512: the 1 taken off before the scaled table value is
 // rounded, so that small x keep their relative accuracy
-__device__ __forceinline__ double expm1(double x)
+static __device__ __noinline__ double expm1_tang(double x)
 {
-    if (!exp_in_range(x)) return ::expm1(x);
     const double t = fma(x, k64OverLn2, kShift);
     const double kd = t - kShift;
     const int k = __double2loint(t);
@@ -111,7 +76,7 @@ __device__ __forceinline__ double log1p_small(double r)
 }
 
 // ln x for finite positive normal x
-__device__ __forceinline__ double log(double x)
+static __device__ __noinline__ double log_tang(double x)
 {
     const int hx = __double2hiint(x), lx = __double2loint(x);
     const int ex = (hx >> 20) & 0x7FF;
@@ -134,11 +99,203 @@ __device__ __forceinline__ double log(double x)
 
 // ln(1 + z) for z > -1: ln u of the rounded u = 1 + z, plus the rounding
 // error of u over u (a tiny correction, taken with a single-precision 1/u)
-__device__ __forceinline__ double log1p(double z)
+static __device__ __noinline__ double log1p_tang(double z)
 {
     const double u = 1.0 + z;
     const double c = z - (u - 1.0);
-    return log(u) + c * (double)__frcp_rn((float)u);
+    return log_tang(u) + c * (double)__frcp_rn((float)u);
 }
+
+// ------------------------------------------------ integer-pipe forms
+// the general operations, out of line: reached by zeros, infinities, NaN,
+// subnormals and results near the ends of the range
+static __device__ __noinline__ double slow_div(double a, double b) { return a / b; }
+static __device__ __noinline__ double slow_sqrt(double x) { return ::sqrt(x); }
+static __device__ __noinline__ double slow_exp(double x) { return ::exp(x); }
+static __device__ __noinline__ double slow_expm1(double x) { return ::expm1(x); }
+static __device__ __noinline__ double slow_pow(double x, double y) { return ::pow(x, y); }
+
+__device__ __forceinline__ double rcp(double x)
+{
+    const uint64_t b = i64::bits(x);
+    const uint32_t e = i64::expo(b);
+    if (e - 1u >= 2044u) return slow_div(1.0, x);
+    const uint64_t r = i64::pack_bits(i64::rcp_m(i64::signif(b)), 1022 - (int)e);
+    return i64::from_bits(r | (b & 0x8000000000000000ull));
+}
+
+__device__ __forceinline__ double div(double a, double b)
+{
+    const uint64_t ba = i64::bits(a), bb = i64::bits(b);
+    const uint32_t ea = i64::expo(ba), eb = i64::expo(bb);
+    if (ea - 1u >= 2046u || eb - 1u >= 2046u || ea - eb + 1000u > 2000u) return slow_div(a, b);
+    uint64_t q = i64::mulhi(i64::signif(ba), i64::rcp_m(i64::signif(bb)));   // in (2^62, 2^64)
+    int e = (int)ea - (int)eb;
+    if (!(q >> 63)) {
+        q <<= 1;
+        --e;
+    }
+    return i64::from_bits(i64::pack_bits(q, e) | ((ba ^ bb) & 0x8000000000000000ull));
+}
+
+__device__ __forceinline__ double sqrt(double x)
+{
+    const uint64_t b = i64::bits(x);
+    const uint32_t e = (uint32_t)(b >> 52);   // with the sign bit: negative x leaves the range
+    if (e - 1u >= 2046u) return slow_sqrt(x);
+    // x = X 2^(2 h), X in [1/4, 1): the significand halved (e even: an odd power of two) or quartered
+    const uint64_t X = i64::signif(b) >> (e & 1u);
+    const uint64_t s = i64::mulhi(X, i64::rsqrt_m(X)) << 1;
+    const int h = ((int)e - 1022 + (int)(e & 1u)) / 2;   // even numerator
+    return i64::from_bits(i64::pack_bits(s, h - 1));
+}
+
+// 2^-(n + F / 2^64), rounded; |n| <= 1000
+__device__ __forceinline__ double pack_exp2_neg(int n, uint64_t F)
+{
+    const uint64_t r = i64::exp2_neg(F);   // units 2^-63, in (2^62, 2^63]
+    const uint64_t q = (r >> 10) + ((r >> 9) & 1u);
+    return i64::from_bits(q + ((uint64_t)(uint32_t)(1021 - n) << 52));
+}
+
+// -x log2(e) = n + F / 2^64 for 2^-60 <= |x| < 64 (biased exponent e)
+__device__ __forceinline__ int exp_arg(uint64_t b, uint32_t e, uint64_t &F)
+{
+    const uint64_t p = i64::mulhi(i64::signif(b), kI64Log2E);   // |x| log2 e = p 2^(e - 1023 - 62)
+    const int s = 1085 - (int)e;                                   // 57..: bits of p below the point
+    int n = 0;
+    if (s >= 64) {
+        F = p >> (s - 64);
+    } else {
+        F = p << (64 - s);
+        n = (int)(p >> s);
+    }
+    if (!(b >> 63)) {   // x > 0: -(n + F)
+        n = -n - (F != 0);
+        F = 0 - F;
+    }
+    return n;
+}
+
+__device__ __forceinline__ double exp(double x)
+{
+    const uint64_t b = i64::bits(x);
+    const uint32_t e = i64::expo(b);
+    if (e - 963u >= 66u) return slow_exp(x);   // |x| outside [2^-60, 64)
+    uint64_t F;
+    const int n = exp_arg(b, e, F);
+    return pack_exp2_neg(n, F);
+}
+
+__device__ __forceinline__ double expm1(double x)
+{
+    const uint64_t b = i64::bits(x);
+    const uint32_t e = i64::expo(b);
+    if (e - 1016u >= 13u) return e >= 1029u ? slow_expm1(x) : expm1_tang(x);   // |x| outside [2^-7, 64)
+    uint64_t F;
+    const int n = exp_arg(b, e, F);
+    const uint64_t r = i64::exp2_neg(F);   // e^x = r 2^-(63 + n)
+    uint64_t d;
+    int ex;   // |result| = d 2^(ex - 63)
+    if (b >> 63) {   // n >= 0: 1 - e^x
+        d = 0x8000000000000000ull - (n < 64 ? r >> n : 0);
+        ex = 0;
+    } else {         // n < 0: e^x - 1, in units of 2^(-63 - n)
+        d = r - (-n < 64 ? 0x8000000000000000ull >> -n : 0);
+        ex = -n;
+    }
+    const int z = __clzll((long long)d);
+    return i64::from_bits(i64::pack_bits(d << z, ex - z) | (b & 0x8000000000000000ull));
+}
+
+// ln of m 2^E with m = M / 2^63 in [1, 2); |ln| at least about 2^-6
+__device__ __forceinline__ double ln_parts(uint64_t M, int E)
+{
+    uint64_t l = i64::log2_m(M);
+    const bool neg = E < 0;
+    if (neg) {   // |E + l| = (-E - 1) + (1 - l)
+        E = -E - (l != 0);
+        l = 0 - l;
+    }
+    // E + l as a normalised 64-bit number v 2^(k - 63)
+    const int k = E ? 31 - __clz(E) : -1 - __clzll((long long)l);
+    const uint64_t v = E ? ((uint64_t)(uint32_t)E << (63 - k)) | (l >> (k + 1)) : l << (-1 - k);
+    uint64_t q = i64::mulhi(v, kI64Ln2);   // in (2^62, 2^64)
+    int e = k;
+    if (!(q >> 63)) {
+        q <<= 1;
+        --e;
+    }
+    return i64::from_bits(i64::pack_bits(q, e) | (neg ? 0x8000000000000000ull : 0));
+}
+
+__device__ __forceinline__ double log(double x)
+{
+    const uint64_t b = i64::bits(x);
+    const uint32_t e = (uint32_t)(b >> 52);
+    // x within [1 - 2^-5, 1 + 2^-5), or not a positive normal number
+    const uint64_t d = b - 0x3FEF000000000000ull;
+    if (e - 1u >= 2046u || d < 0x0001800000000000ull) return log_tang(x);
+    return ln_parts(i64::signif(b), (int)e - 1023);
+}
+
+__device__ __forceinline__ double log1p(double z)
+{
+    const uint64_t b = i64::bits(z);
+    const uint32_t e = (uint32_t)(b >> 52);
+    if (e - 1018u >= 57u) return log1p_tang(z);   // z outside [2^-5, 2^52)
+    // 1 + z, exact in 64 bits
+    uint64_t M = i64::signif(b);
+    int E = (int)e - 1023;
+    if (E < 0) {
+        M = 0x8000000000000000ull + (M >> -E);
+        E = 0;
+    } else {
+        const uint64_t s = M + (0x8000000000000000ull >> E);
+        const bool carry = s < M;
+        M = carry ? (s >> 1) | 0x8000000000000000ull : s;
+        E += carry;
+    }
+    return ln_parts(M, E);
+}
+
+// x^-b in units of 2^-64 for the bits of a normal x with x^-b below 1, b = B / 2^64
+__device__ __forceinline__ uint64_t pow_frac_fixed(uint64_t bx, uint64_t B)
+{
+    const uint32_t E = (uint32_t)(bx >> 52) - 1023u;   // x >= 1: E >= 0
+    const uint64_t w0 = i64::wide(i64::lo32(B), E), w1 = i64::wide(i64::hi32(B), E) + (w0 >> 32);
+    const uint64_t F = (w1 << 32) | i64::lo32(w0);
+    const uint64_t G = F + i64::mulhi(i64::log2_m(i64::signif(bx)), B);
+    const uint32_t n = (uint32_t)(w1 >> 32) + (G < F);
+    return (i64::exp2_neg(G) << 1) >> n;
+}
+
+// x^-b (or, NEG = false, x^b) for a positive normal x and b = B / 2^64 in (0, 1)
+template <bool NEG>
+__device__ __forceinline__ double pow_frac(double x, uint64_t B)
+{
+    const uint64_t bx = i64::bits(x);
+    const uint32_t e = (uint32_t)(bx >> 52);
+    if (e - 1u >= 2046u) return slow_pow(x, (NEG ? -5.421010862427522e-20 : 5.421010862427522e-20) * (double)B);
+    // b log2 x = b E + b l
+    const int E = (int)e - 1023;
+    const uint32_t a = (uint32_t)(E < 0 ? -E : E);
+    const uint64_t w0 = i64::wide(i64::lo32(B), a), w1 = i64::wide(i64::hi32(B), a) + (w0 >> 32);
+    uint64_t F = (w1 << 32) | i64::lo32(w0);
+    int n = (int)(w1 >> 32);
+    if (E < 0) {
+        n = -n - (F != 0);
+        F = 0 - F;
+    }
+    uint64_t G = F + i64::mulhi(i64::log2_m(i64::signif(bx)), B);
+    n += G < F;
+    if (!NEG) {
+        n = -n - (G != 0);
+        G = 0 - G;
+    }
+    return pack_exp2_neg(n, G);
+}
+__device__ __forceinline__ double pow_neg(double x, uint64_t B) { return pow_frac<true>(x, B); }
+__device__ __forceinline__ double cbrt(double x) { return pow_frac<false>(x, 0x5555555555555555ull); }   // x >= 0
 
 }  // namespace m64
