@@ -61,6 +61,10 @@ struct pr_ctx {
     float *d_corr32;
     int corr_nT, corr_nP;
     int occ_species[2];  // [FP64, FP32]
+    // tables of the fixed-point FP64 kernel (pr_species.cu SpFix9), or NULL
+    // when a constant leaves its range; its resident blocks per SM
+    void *h_spfix;
+    int occ_spfix;
     // Bilger's mixture fraction: per-species coefficients b_k of the coupling
     // function, then beta_ox and 1 / (beta_fuel - beta_ox) ([n_species + 2])
     double *d_bilger64;

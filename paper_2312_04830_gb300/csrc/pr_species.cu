@@ -30,6 +30,7 @@
 
 #include <cmath>
 #include <cstring>
+#include <new>
 #include <vector>
 
 #include "pr_device.cuh"
@@ -103,7 +104,7 @@ __global__ void __launch_bounds__(kSpBlock) species_kernel(const SpArgs<Real> a)
             continue;
         }
         if (a.hk) {
-            const Real iRT = Real(1) / (Real(prk::kR) * T);
+            const Real iRT = M<Real>::rcp(Real(prk::kR) * T);
 #pragma unroll
             for (int k = 0; k < NS; ++k) {
                 if (k >= a.N) break;
@@ -111,7 +112,7 @@ __global__ void __launch_bounds__(kSpBlock) species_kernel(const SpArgs<Real> a)
             }
         }
         if (a.Dk) {
-            const Real inv_s = Real(1) / s;
+            const Real inv_s = M<Real>::rcp(s);
 #pragma unroll
             for (int k = 0; k < NS; ++k) x[k] *= inv_s;
             Real D[NS];
@@ -121,6 +122,147 @@ __global__ void __launch_bounds__(kSpBlock) species_kernel(const SpArgs<Real> a)
                 if (k >= a.N) break;
                 a.Dk[(int64_t)k * a.ldo + i] = D[k];
             }
+        }
+    }
+}
+
+// The FP64 outputs of up to 9 species without a correction table: the pair
+// sums in fixed point (pr_species.cuh), every table in the kernel's parameter
+// space, cells outside the fixed-point range through the general form.
+// D_k = (sum_{j != k} y_j / sum_j y_j) f T^1.5 / p / sum_{j != k} x_j / D_kj p / T^1.5
+// with moles per kg n_j = y_j / W_j in place of x_j = n_j / sum n (one factor
+// per cell); h_k / (R T) = sum_j a_j T^j / (j + 1) + a_6 / T.
+struct SpFix9 {
+    prs::OmegaFix om[prs::kPairs9];     // of each distinct eps
+    prs::PairFix pair[prs::kPairs9];    // ordered by eps
+    int32_t first[prs::kPairs9 + 1];    // a distinct eps's first pair
+    int32_t n_om;
+    double h[2][9][6];        // a_1, a_2/2, ..., a_5/5, a_6 of the low and the high range
+    double tmid[9], iW[9];
+};
+
+static __device__ __noinline__ void diffusion_general9(const double *y9, const double *x9, double ysum, double T,
+                                                       double p, int N, const double *tab, const double *corr, int cT,
+                                                       int cP, double *D9)
+{
+    double y[9], x[9], D[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        y[k] = y9[k];
+        x[k] = x9[k];
+    }
+    prs::diffusion_cell<double, 9>(y, x, ysum, T, p, N, tab, corr, cT, cP, D);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) D9[k] = D[k];
+}
+
+__global__ void __launch_bounds__(kSpBlock, 6) species_fix_kernel(const __grid_constant__ SpArgs<double> a,
+                                                               const __grid_constant__ SpFix9 t)
+{
+    __shared__ uint64_t s_exp2[1024];
+    __shared__ double s_x[9][kSpBlock], s_acc[9][kSpBlock];   // this thread's columns: no barrier between uses
+    if (a.Dk) {
+        for (int e = threadIdx.x; e < 512; e += blockDim.x)
+            reinterpret_cast<ulonglong2 *>(s_exp2)[e] = reinterpret_cast<const ulonglong2 *>(kI64Exp2)[e];
+        __syncthreads();
+    }
+    const double nanv = M<double>::nan();
+    const int tid = threadIdx.x, N = a.N;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + tid; i < a.n; i += stride) {
+        const double T = __ldg(a.T + i), p = __ldg(a.p + i);
+        double y[9];
+        double ysum = 0, s = 0;
+        bool ok = (T > 0.0) && (p > 0.0) && M<double>::finite(T) && M<double>::finite(p);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) y[k] = (k < N) ? __ldg(a.Y + (int64_t)k * a.ldY + i) : 0.0;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            ok = ok && prk::nonneg_finite(y[k]);
+            ysum += y[k];
+            const double x = y[k] * t.iW[k];
+            s_x[k][tid] = x;
+            s_acc[k][tid] = 0.0;
+            s += x;
+        }
+        ok = ok && (M<double>::fabs(ysum - 1.0) <= 1e-6) && (s > 0.0);
+        if (a.status) a.status[i] = ok ? prk::kOk : prk::kBadInput;
+        if (!ok) {
+            for (int k = 0; k < N; ++k) {
+                if (a.hk) a.hk[(int64_t)k * a.ldo + i] = nanv;
+                if (a.Dk) a.Dk[(int64_t)k * a.ldo + i] = nanv;
+            }
+            continue;
+        }
+        if (a.hk) {
+            const double iT = M<double>::rcp(T);
+#pragma unroll 1
+            for (int k = 0; k < N; ++k) {
+                const bool low = prk::lt_pos(T, t.tmid[k]);
+                const double *e = t.h[low ? 0 : 1][k];
+                const double h = fma(fma(fma(fma(e[4], T, e[3]), T, e[2]), T, e[1]), T, e[0]);
+                a.hk[(int64_t)k * a.ldo + i] = fma(e[5], iT, h);
+            }
+        }
+        if (!a.Dk) continue;
+        if (!prs::fix_range(T)) {
+            const double inv_s = M<double>::rcp(s);
+            double x[9], D[9];
+#pragma unroll
+            for (int k = 0; k < 9; ++k) x[k] = s_x[k][tid] * inv_s;
+            diffusion_general9(y, x, ysum, T, p, N, a.dtab, a.corr, 0, 0, D);
+            for (int k = 0; k < N; ++k) a.Dk[(int64_t)k * a.ldo + i] = D[k];
+            continue;
+        }
+        // s T^(3/2) / (p sum_j y_j)
+        const double scale = M<double>::div(s * T * M<double>::sqrt(T), p * ysum);
+        const uint64_t bT = i64::bits(T);
+        const uint64_t Tf = i64::signif(bT) >> (1035u - (uint32_t)(bT >> 52));
+        const uint64_t TB = m64::pow_frac_fixed(bT, (uint64_t)(prs::kNB * 18446744073709551616.0));
+        // in loops: unrolled, their ~6000 instructions miss the instruction
+        // cache (the accumulators then live in shared memory)
+#pragma unroll 1
+        for (int u = 0; u < t.n_om; ++u) {
+            const uint64_t om = prs::omega_fix(t.om[u], Tf, TB, s_exp2);
+#pragma unroll 1
+            for (int q = t.first[u]; q < t.first[u + 1]; ++q) {
+                const double w = prs::pair_fix(t.pair[q], om);
+                const int k = t.pair[q].k, j = t.pair[q].j;
+                s_acc[k][tid] = fma(s_x[j][tid], w, s_acc[k][tid]);
+                s_acc[j][tid] = fma(s_x[k][tid], w, s_acc[j][tid]);
+            }
+        }
+        // (y read again: held across the pairs it would cost 18 registers)
+#pragma unroll
+        for (int k = 0; k < 9; ++k) y[k] = (k < N) ? __ldg(a.Y + (int64_t)k * a.ldY + i) : 0.0;
+        // sum_{j != k} y_j from prefix and suffix sums
+        double others[9];
+        double run = 0;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            others[k] = run;
+            run += y[k];
+        }
+        run = 0;
+#pragma unroll
+        for (int k = 8; k >= 0; --k) {
+            others[k] += run;
+            run += y[k];
+        }
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            if (k >= N) break;
+            const double acc = s_acc[k][tid];
+            double D;
+            if (acc > 0.0) {
+                D = M<double>::div(others[k] * scale, acc);
+            } else {   // alone in the cell: self-diffusion, the general form
+                const double *ie = a.dtab + 18, *epsB = ie + 81, *ic = epsB + 81;
+                const double TmB = prk::pow_neg<double>(T, prs::kNB);
+                D = M<double>::div(M<double>::div(T * M<double>::sqrt(T), p),
+                                   prs::omega_d<double>(T * ie[10 * k], TmB * epsB[10 * k]) * ic[10 * k]);
+            }
+            a.Dk[(int64_t)k * a.ldo + i] = D;
         }
     }
 }
@@ -160,6 +302,58 @@ int occ_of()
 
 namespace prgb {
 
+// The fixed-point kernel's tables; false where a pair constant leaves its
+// range (eps_kj below 22.5 K, or a collision integral above 4 at 32 K).
+static bool fill_fix9(SpFix9 &f, const pr_species_table *tbl)
+{
+    typedef long double ld;   // at least 64 significant bits on x86-64 and aarch64
+    const int N = tbl->n_species;
+    std::memset(&f, 0, sizeof(f));
+    const ld log2e = 1.442695040888963407359924681001892137L;
+    const ld D[3] = {(ld)prs::kND, (ld)prs::kNF, (ld)prs::kNH};
+    for (int k = 0; k < N; ++k) {
+        f.tmid[k] = tbl->T_mid[k];
+        f.iW[k] = 1.0 / (tbl->W[k] * 1e-3);
+        for (int j = 0; j < 6; ++j) {
+            f.h[0][k][j] = j < 5 ? tbl->nasa_lo[7 * k + j] / (j + 1) : tbl->nasa_lo[7 * k + 5];
+            f.h[1][k][j] = j < 5 ? tbl->nasa_hi[7 * k + j] / (j + 1) : tbl->nasa_hi[7 * k + 5];
+        }
+    }
+    // the distinct eps_kj^2 ~ Tc_k Tc_j, in order of first appearance, and their pairs
+    int n_pair = 0;
+    bool seen[9][9] = {};
+    for (int k0 = 0; k0 < N; ++k0)
+        for (int j0 = k0 + 1; j0 < N; ++j0) {
+            if (seen[k0][j0]) continue;
+            const ld e2 = (ld)tbl->Tc[k0] * (ld)tbl->Tc[j0], eps = sqrtl(e2) / 1.2593L;
+            const ld pw = 0.5L * (ld)prs::kNA * powl(eps, (ld)prs::kNB);
+            // Omega_D / 2 at 32 K, its largest, within the sum's four units (and A eps^B / 2 below 2)
+            if (!(eps > 22.5L) || !(pw < 2.0L) || !(pw * powl(32.0L, -(ld)prs::kNB) < 2.4L)) return false;
+            prs::OmegaFix &o = f.om[f.n_om];
+            for (int m = 0; m < 3; ++m) o.a[m] = (uint64_t)roundl(ldexpl(D[m] * log2e / eps, 66));
+            o.pw = (uint64_t)roundl(ldexpl(pw, 63));
+            f.first[f.n_om++] = n_pair;
+            for (int k = k0; k < N; ++k)
+                for (int j = k + 1; j < N; ++j) {
+                    if (seen[k][j] || (ld)tbl->Tc[k] * (ld)tbl->Tc[j] != e2) continue;
+                    seen[k][j] = true;
+                    const ld sig = 0.5L * 0.809L * (cbrtl((ld)tbl->Vc[k]) + cbrtl((ld)tbl->Vc[j]));
+                    const ld Mkj = 2.0L / (1.0L / (ld)tbl->W[k] + 1.0L / (ld)tbl->W[j]);
+                    int e;
+                    const ld fr = frexpl(sqrtl(Mkj) * sig * sig / 0.0266L, &e);   // 1 / c_kj = fr 2^e, fr in [1/2, 1)
+                    const ld m64 = roundl(ldexpl(fr, 64));
+                    if (!(m64 < 18446744073709551616.0L) || e < -900 || e > 900) return false;
+                    f.pair[n_pair].icm = (uint64_t)m64;
+                    f.pair[n_pair].ice = e - 1;
+                    f.pair[n_pair].k = (uint16_t)k;
+                    f.pair[n_pair].j = (uint16_t)j;
+                    ++n_pair;
+                }
+        }
+    f.first[f.n_om] = n_pair;
+    return true;
+}
+
 // Pair constants from the validated species table (entries of species >= N
 // are zero and never read).
 pr_status species_tables_init(pr_ctx *c, const pr_species_table *tbl)
@@ -182,6 +376,15 @@ pr_status species_tables_init(pr_ctx *c, const pr_species_table *tbl)
             epsB[k * NS + j] = std::pow(eps, prs::kNB);
             ic[k * NS + j] = 1.0 / ckj;
         }
+    if (NS == 9) {
+        SpFix9 *f = new (std::nothrow) SpFix9();
+        if (!f) {
+            set_error("pr_create: host allocation failed");
+            return PR_ENOMEM;
+        }
+        if (fill_fix9(*f, tbl)) c->h_spfix = f;
+        else delete f;
+    }
     std::vector<float> t32(t.size());
     for (size_t e = 0; e < t.size(); ++e) t32[e] = (float)t[e];
     PR_CUDA_TRY(cudaMalloc(&c->d_dtab64, t.size() * sizeof(double)));
@@ -195,6 +398,9 @@ pr_status species_tables_init(pr_ctx *c, const pr_species_table *tbl)
     PR_CUDA_TRY(cudaMemcpy(c->d_dtab32, t32.data(), t32.size() * sizeof(float), cudaMemcpyHostToDevice));
     c->corr_nT = c->corr_nP = 0;
     c->occ_species[0] = (NS == 9) ? occ_of<double, 9>() : occ_of<double, 32>();
+    c->occ_spfix = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c->occ_spfix, species_fix_kernel, kSpBlock, 0);
+    c->occ_spfix = c->occ_spfix > 0 ? c->occ_spfix : 1;
     c->occ_species[1] = (NS == 9) ? occ_of<float, 9>() : occ_of<float, 32>();
     return PR_OK;
 }
@@ -207,6 +413,7 @@ void species_tables_free(pr_ctx *c)
     cudaFree(c->d_corr32);
     cudaFree(c->d_bilger64);
     cudaFree(c->d_bilger32);
+    delete static_cast<SpFix9 *>(c->h_spfix);
 }
 
 }  // namespace prgb
@@ -330,7 +537,12 @@ pr_status pr_species_props(pr_ctx *ctx, pr_precision prec, int64_t n, const void
         SpArgs<double> a{n, ldY, ldo, (const double *)T, (const double *)p, (const double *)Y, (double *)hk_RT,
                          (double *)Dk, cell_status, (const SpeciesRec<double> *)ctx->d_sp64, ctx->d_dtab64,
                          ctx->d_corr64, ctx->n_species, ctx->corr_nT, ctx->corr_nP};
-        if (nine) launch_species<double, 9>(a, ctx->occ_species[0], ctx->num_sms, st);
+        // the fixed-point kernel: tables within its ranges, no correction table
+        if (nine && ctx->h_spfix && ctx->corr_nT == 0) {
+            const int64_t need = (n + kSpBlock - 1) / kSpBlock, cap = (int64_t)ctx->occ_spfix * ctx->num_sms;
+            species_fix_kernel<<<(int)(need < cap ? need : cap), kSpBlock, 0, st>>>(
+                a, *static_cast<const SpFix9 *>(ctx->h_spfix));
+        } else if (nine) launch_species<double, 9>(a, ctx->occ_species[0], ctx->num_sms, st);
         else launch_species<double, 32>(a, ctx->occ_species[0], ctx->num_sms, st);
     } else {
         SpArgs<float> a{n, ldY, ldo, (const float *)T, (const float *)p, (const float *)Y, (float *)hk_RT,

@@ -22,9 +22,11 @@ constexpr double kNE = 1.03587, kNF = 1.52996, kNG = 1.76474, kNH = 3.89411;
 // Flat per-context table: tc[NS], pc[NS], ie[NS*NS], epsB[NS*NS], ic[NS*NS].
 inline size_t dtab_len(int NS) { return 2 * (size_t)NS + 3 * (size_t)NS * NS; }
 
-// Omega_D at T* = Ts, with pw = T*^-B given.
+// Omega_D at T* = Ts, with pw = T*^-B given.  In FP64 this is the general
+// form, out of line (36 copies of it would fill the instruction cache); the
+// usual temperatures take the fixed-point form below.
 template <typename Real>
-__device__ __forceinline__ Real omega_d(Real Ts, Real pw)
+__device__ __forceinline__ Real omega_d_inline(Real Ts, Real pw)
 {
     Real om = Real(kNA) * pw;
     if (Ts < Real(40.0 / kND)) om = M<Real>::fma(Real(kNC), M<Real>::exp(Real(-kND) * Ts), om);
@@ -33,7 +35,71 @@ __device__ __forceinline__ Real omega_d(Real Ts, Real pw)
     return om;
 }
 
-// Bilinear, clamped to the table's edges.
+static __device__ __noinline__ double omega_d_f64(double Ts, double pw) { return omega_d_inline<double>(Ts, pw); }
+
+template <typename Real>
+__device__ __forceinline__ Real omega_d(Real Ts, Real pw)
+{
+    if constexpr (sizeof(Real) == 8)
+        return omega_d_f64(Ts, pw);
+    else
+        return omega_d_inline<Real>(Ts, pw);
+}
+
+// ------------------------------------------------ fixed-point pair sums
+// For T in [32, 8192) K the pair sums sum_{j != k} n_j / c_kj Omega_kj take
+// Omega_D from the integer pipe (pr_int64.cuh).  T is exact in units of
+// 2^-51 K; each exponential's argument T D log2(e) / eps_kj is one 64-bit
+// product, in units of 2^-53, with log2 of its factor (C, E, G) and of the
+// common 1/2 added, so that a term is 2^-argument; Omega_D / 2 is summed in
+// units of 2^-62 and leaves as a double after the product with 1 / c_kj.
+// Truncations add up to at most 3 x 2^-53 of an argument (0.25 of the sum's
+// rounding at the largest share the exponentials take of Omega_D) and
+// 2^-60 of the sum.  Per Omega_D ~150 integer instructions replace ~45 FP64
+// ones, which hold the FP64 pipe 16 cycles each.
+// Omega_D depends on a pair through eps_kj alone, so pairs of equal eps (the
+// radicals take their parent molecule's critical constants) share one: 21 for
+// the 36 pairs of the nine species here.
+struct OmegaFix {
+    uint64_t a[3];    // D, F, H log2(e) / eps, units 2^-66 (below 1/4)
+    uint64_t pw;      // A eps^B / 2, units 2^-63 (below 2)
+};
+struct PairFix {
+    uint64_t icm;     // 1 / c_kj = icm 2^(ice - 63), icm normalised
+    int32_t ice;
+    uint16_t k, j;
+};
+constexpr int kPairs9 = 36;
+
+// 1 - log2 of C, E, G in units of 2^-53, plus one unit for the truncations
+constexpr uint64_t kOffC = 0x006BF24BFBC86A2Bull, kOffE = 0x001E5F7E967FD2C7ull, kOffG = 0x0005C704F3E28E63ull;
+
+// Omega_D / 2 in units of 2^-62: Tf = T 2^51, TB = T^-B 2^64; tab: kI64Exp2 (a copy).
+__device__ __forceinline__ uint64_t omega_fix(const OmegaFix &c, uint64_t Tf, uint64_t TB, const uint64_t *tab)
+{
+    uint64_t om = i64::mulhi(TB, c.pw) >> 1;
+    const uint64_t p0 = i64::mulhi(Tf, c.a[0]) + kOffC;
+    const uint64_t p1 = i64::mulhi(Tf, c.a[1]) + kOffE;
+    const uint64_t p2 = i64::mulhi(Tf, c.a[2]) + kOffG;
+    // a term of 2^-62 or less of the sum's units is dropped
+    const uint32_t n0 = i64::hi32(p0) >> 21, n1 = i64::hi32(p1) >> 21, n2 = i64::hi32(p2) >> 21;
+    if (n0 < 62) om += i64::exp2_neg(p0 << 11, tab) >> (n0 + 1u);
+    if (n1 < 62) om += i64::exp2_neg(p1 << 11, tab) >> (n1 + 1u);
+    if (n2 < 62) om += i64::exp2_neg(p2 << 11, tab) >> (n2 + 1u);
+    return om;
+}
+
+// Omega_D / c_kj
+__device__ __forceinline__ double pair_fix(const PairFix &c, uint64_t om)
+{
+    const uint64_t q = i64::mulhi(om, c.icm);
+    const int z = __clzll((long long)q);
+    return i64::from_bits(i64::pack_bits(q << z, c.ice + 3 - z));
+}
+
+// Whether T lies in the fixed-point range [32, 8192) K
+__device__ __forceinline__ bool fix_range(double T) { return (i64::bits(T) >> 52) - 1028u < 8u; }
+
 template <typename Real>
 __device__ __forceinline__ Real corr_factor(const Real *__restrict__ c, int cT, int cP, Real x, Real y)
 {
@@ -66,7 +132,7 @@ __device__ __forceinline__ void diffusion_cell(const Real (&y)[NS], const Real (
         ppc = M<Real>::fma(x[k], pc[k], ppc);
     }
     const Real f = (cT > 0) ? corr_factor<Real>(corr, cT, cP, T / Tpc, p / ppc) : Real(1);
-    const Real TmB = M<Real>::exp(Real(-kNB) * M<Real>::log(T));   // T^-B
+    const Real TmB = prk::pow_neg<Real>(T, kNB);   // T^-B
     Real acc[NS];
 #pragma unroll
     for (int k = 0; k < NS; ++k) acc[k] = 0;
@@ -83,7 +149,7 @@ __device__ __forceinline__ void diffusion_cell(const Real (&y)[NS], const Real (
             acc[j] = M<Real>::fma(x[k], w, acc[j]);
         }
     }
-    const Real scale = f * T * M<Real>::sqrt(T) / p;   // f T^(3/2) / p
+    const Real scale = M<Real>::div(f * T * M<Real>::sqrt(T), p);   // f T^(3/2) / p
     // sum_{j != k} y_j from prefix and suffix sums
     Real others[NS];
     Real run = 0;
@@ -98,15 +164,15 @@ __device__ __forceinline__ void diffusion_cell(const Real (&y)[NS], const Real (
         others[k] += run;
         run += y[k];
     }
-    const Real iys = Real(1) / ysum;
+    const Real iys = M<Real>::rcp(ysum);
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
         if (k >= N) break;
         if (acc[k] > Real(0)) {
-            D[k] = others[k] * iys * scale / acc[k];
+            D[k] = M<Real>::div(others[k] * iys * scale, acc[k]);
         } else {   // alone in the cell: self-diffusion
             const int q = k * NS + k;
-            D[k] = scale / (omega_d<Real>(T * ie[q], TmB * epsB[q]) * ic[q]);
+            D[k] = M<Real>::div(scale, omega_d<Real>(T * ie[q], TmB * epsB[q]) * ic[q]);
         }
     }
 }
