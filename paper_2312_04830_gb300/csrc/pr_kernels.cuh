@@ -269,13 +269,14 @@ __device__ __forceinline__ bool one_step_ok(const FirstEval &f, double T, double
     return clear;
 }
 
-// h(T) and cp(T) in FP32 with FP32 arguments (the warm start's evaluations).
-template <int NS, bool KIJ>
+// h(T) and cp(T) in FP32 with FP32 arguments (the warm start's evaluations,
+// and the FP32 and mixed inversions').
+template <int NS, bool KIJ, typename RZ = float>
 __device__ __noinline__ int eval_h_f32(const Comp<float, NS> &c, float T, float p, const SpeciesRec<float> *sp,
                                        const float *kij, float tmid_u, float &h, float &cp)
 {
     Thermo<float> th;
-    thermo<float, float, NS, KIJ>(c, T, p, sp, kij, th, tmid_u);
+    thermo<float, RZ, NS, KIJ>(c, T, p, sp, kij, th, tmid_u);
     if (th.status == kNoRoot) return kNoRoot;
     h = th.h;
     cp = th.cp;
@@ -379,9 +380,84 @@ __device__ __forceinline__ int newton_solve(const Comp<Real, NS> &c, double hs, 
     return st;
 }
 
+// A temperature as an unevaluated sum of two floats, h = the sum rounded.
+struct Temp2 {
+    float h, l;
+};
+__device__ __forceinline__ Temp2 temp2_add(Temp2 a, float b)
+{
+    // two-sum of h and b (Knuth), the tail added and the result renormalised
+    const float s = __fadd_rn(a.h, b), bb = __fsub_rn(s, a.h);
+    const float e = __fadd_rn(__fadd_rn(__fsub_rn(a.h, __fsub_rn(s, bb)), __fsub_rn(b, bb)), a.l);
+    const float h = __fadd_rn(s, e);
+    return {h, __fsub_rn(e, __fsub_rn(h, s))};
+}
+__device__ __forceinline__ bool temp2_less(Temp2 a, Temp2 b) { return a.h < b.h || (a.h == b.h && a.l < b.l); }
+
+// newton_solve for the FP32 and mixed inversions, its bookkeeping in FP32: T
+// as a two-float number (48 bits; h(T) is evaluated at its rounded value
+// anyway), the residual h - h* of two FP32 numbers, the step's quotient and
+// the tests in FP32.  In double, these ~25 FP64-pipe operations per iteration
+// (77 per cell) held the FP32 kernel, the pipe 80 % busy and the issue slots
+// 44 %: 4.5 M cells of the flame field 703 us (535 us with the division on
+// the integer pipe), 365 us with this bookkeeping, errors unchanged.
+template <typename RZ, int NS, bool KIJ>
+__device__ __forceinline__ int newton_solve_f32(const Comp<float, NS> &c, float hs, float p, float T0,
+                                                const SpeciesRec<float> *sp, const float *kij, float tmid_u,
+                                                int max_iter, float rtol, float jump_tol, Temp2 &Tres, int &iters,
+                                                float &cp_last)
+{
+    const float tlo = (float)kTLo, thi = (float)kTHi;
+    Temp2 lo = {tlo, 0.f}, hi = {thi, 0.f}, t = {T0, 0.f};
+    bool lo_done = false, hi_done = false;   // endpoint h evaluated (range checked)
+    float fprev = INFINITY;
+    int st = kMaxIt, it;
+    Tres = t;
+    cp_last = 0.f;
+#pragma unroll 1
+    for (it = 1; it <= max_iter; ++it) {
+        float h, cp;
+        const int e = eval_h_f32<NS, KIJ, RZ>(c, t.h, p, sp, kij, tmid_u, h, cp);
+        if (e) { st = e; Tres = t; break; }
+        cp_last = cp;
+        const float f = h - hs;
+        if (fabsf(f) <= rtol * fmaxf(fabsf(hs), fabsf(cp) * t.h)) { st = kOk; Tres = t; break; }
+        if (f < 0) lo = t; else hi = t;
+        Temp2 tn = temp2_add(t, -(f / cp));
+        const bool newton_ok = (cp > 0) && temp2_less(lo, tn) && temp2_less(tn, hi) && (fabsf(f) <= 0.5f * fabsf(fprev));
+        if (!newton_ok) {
+            tn = temp2_add(temp2_add(lo, hi.h), hi.l);
+            tn.h *= 0.5f;
+            tn.l *= 0.5f;
+            if ((lo.h == tlo && lo.l == 0.f && !lo_done) || (hi.h == thi && hi.l == 0.f && !hi_done)) {
+                const bool use_lo = (lo.h == tlo && lo.l == 0.f && !lo_done);
+                const float Te = use_lo ? tlo : thi;
+                float he, cpe;
+                const int e2 = eval_h_f32<NS, KIJ, RZ>(c, Te, p, sp, kij, tmid_u, he, cpe);
+                if (e2) { st = e2; Tres = t; break; }
+                if (use_lo) lo_done = true; else hi_done = true;
+                if ((use_lo && hs < he) || (!use_lo && hs > he)) { st = kHRange; Tres = {Te, 0.f}; break; }
+            }
+        }
+        fprev = f;
+        if (fabsf((tn.h - t.h) + (tn.l - t.l)) <= rtol * t.h) {
+            Tres = tn;
+            float h2, cp2;
+            if (eval_h_f32<NS, KIJ, RZ>(c, tn.h, p, sp, kij, tmid_u, h2, cp2)) { st = kNoRoot; break; }
+            cp_last = cp2;
+            st = (fabsf(h2 - hs) <= jump_tol * fmaxf(fabsf(hs), fabsf(cp2) * tn.h)) ? kOk : kHRange;
+            break;
+        }
+        t = tn;
+        Tres = tn;
+    }
+    iters = it > max_iter ? max_iter : it;
+    return st;
+}
+
 // Mass-specific ideal-gas cp of a cell [J/(kg K)] (NASA-7).
 template <typename Real, int NS>
-__device__ __forceinline__ double cp_ideal_mass(const Comp<Real, NS> &c, Real T, const SpeciesRec<Real> *sp)
+__device__ __forceinline__ Real cp_ideal_mass(const Comp<Real, NS> &c, Real T, const SpeciesRec<Real> *sp)
 {
     Real s = 0;
 #pragma unroll
@@ -390,7 +466,7 @@ __device__ __forceinline__ double cp_ideal_mass(const Comp<Real, NS> &c, Real T,
         const Real cpk = M<Real>::fma(M<Real>::fma(M<Real>::fma(M<Real>::fma(a[4], T, a[3]), T, a[2]), T, a[1]), T, a[0]);
         s = M<Real>::fma(c.x[k], cpk, s);
     }
-    return M<double>::div((double)s, (double)c.Wbar);
+    return M<Real>::div(s, c.Wbar);
 }
 
 // Composition in FP64 from FP32 mass fractions (the FP64 re-solve of the
@@ -530,51 +606,99 @@ __global__ void __launch_bounds__(kBlock) newton_kernel(const NewtonArgs<Real> a
     constexpr bool kMixed = sizeof(Real) == 4 && sizeof(RZ) == 8;
     __shared__ typename std::conditional<kMixed, Smem<double, NS, KIJ>, char>::type s64[1];
     if constexpr (kMixed) stage<double, NS, KIJ>(s64[0], a.sp64, a.pair64, a.kij64);
-    // FP32 thermodynamics resolve h to ~1e-7 of its scale: floor the tolerance
-    const double rtol = (sizeof(Real) == 4) ? fmax(a.rtol, 2e-6) : a.rtol;
-    const double jump_tol = (sizeof(Real) == 4) ? 2e-5 : 1e-6;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     if constexpr (kFp64) {
         if (warm) {
-            newton_fp64_queued<NS, KIJ>(a, s, s32[0], stride, rtol, jump_tol);
+            newton_fp64_queued<NS, KIJ>(a, s, s32[0], stride, a.rtol, 1e-6);
             return;
         }
-    }
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += stride) {
-        const double hs = (double)__ldg(a.hstar + i);
-        const Real p = __ldg(a.p + i);
-        const double Tg = (double)__ldg(a.Tg + i);
-        Comp<Real, NS> c;
-        bool ok = load_comp<Real, NS>(c, a.Y, a.ldY, i, a.N, s.sp);
-        ok = ok && isfinite(hs) && isfinite(Tg) && (p > Real(0)) && M<Real>::finite(p);
-        int st = kBadInput, it = 0;
-        double Tres = nan("");
-        if (ok) {
-            double T = fmin(fmax(Tg, kTLo), kTHi);
-            double cp_last;
-            st = newton_solve<Real, RZ, NS, KIJ>(c, hs, p, T, s.sp, s.kij, (Real)a.tmid_u, a.max_iter, rtol, jump_tol,
-                                                 Tres, it, cp_last);
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += stride) {
+            const double hs = __ldg(a.hstar + i), p = __ldg(a.p + i), Tg = __ldg(a.Tg + i);
+            Comp<double, NS> c;
+            bool ok = load_comp<double, NS>(c, a.Y, a.ldY, i, a.N, s.sp);
+            ok = ok && isfinite(hs) && isfinite(Tg) && (p > 0.0) && isfinite(p);
+            int st = kBadInput, it = 0;
+            double Tres = nan("");
+            if (ok) {
+                double cp_last;
+                st = newton_solve<double, double, NS, KIJ>(c, hs, p, fmin(fmax(Tg, kTLo), kTHi), s.sp, s.kij, a.tmid_u,
+                                                           a.max_iter, a.rtol, 1e-6, Tres, it, cp_last);
+            }
+            a.Tout[i] = Tres;
+            a.status[i] = st;
+            if (a.iters) a.iters[i] = it;
+        }
+    } else {
+        // mixed: cells to be solved again in FP64 wait in a queue of the block
+        // until there is one for every thread, so that FP64 iterations run in
+        // full warps (as in newton_fp64_queued): 300007 scattered cells 289 ->
+        // 203 us, with the bookkeeping above
+        __shared__ int q_n;
+        constexpr int kQ = kMixed ? 2 * kBlock : 1;
+        __shared__ int64_t q_i[kQ];
+        __shared__ float q_h[kQ], q_l[kQ];   // the start, a two-float T
+        __shared__ int q_it[kQ];
+        if (kMixed && threadIdx.x == 0) q_n = 0;
+        if (kMixed) __syncthreads();
+        auto finish = [&](int e) {
             if constexpr (kMixed) {
-                // FP64 where FP32 is least reliable: failed cells, and cells in
-                // the pseudo-boiling band, from the FP32 root (or the guess)
-                const bool band = st == kOk && cp_last > kPseudoCriticalCp * cp_ideal_mass<Real, NS>(c, (Real)Tres, s.sp);
-                if (st != kOk || band) {
-                    Comp<double, NS> c64;
-                    if (comp_fp64_of_fp32<NS>(c64, a.Y, a.ldY, i, a.N, s64[0].sp)) {
-                        const double T0 = (st == kOk) ? Tres : fmin(fmax(Tg, kTLo), kTHi);
-                        double T64, cp64;
-                        int it64;
-                        st = newton_solve<double, double, NS, KIJ>(c64, hs, (double)p, T0, s64[0].sp, s64[0].kij,
-                                                                   a.tmid_u, a.max_iter, a.rtol, 1e-6, T64, it64, cp64);
-                        Tres = T64;
-                        it += it64;
+                const int64_t i = q_i[e];
+                Comp<double, NS> c64;
+                if (comp_fp64_of_fp32<NS>(c64, a.Y, a.ldY, i, a.N, s64[0].sp)) {
+                    double T64, cp64;
+                    int it64;
+                    const int st = newton_solve<double, double, NS, KIJ>(
+                        c64, (double)__ldg(a.hstar + i), (double)__ldg(a.p + i), (double)q_h[e] + (double)q_l[e],
+                        s64[0].sp, s64[0].kij, a.tmid_u, a.max_iter, a.rtol, 1e-6, T64, it64, cp64);
+                    a.Tout[i] = (float)T64;   // over the FP32 result
+                    a.status[i] = st;
+                    if (a.iters) a.iters[i] = q_it[e] + it64;
+                }
+            }
+        };
+        // FP32 thermodynamics resolve h to ~1e-7 of its scale: floor the tolerance
+        const float rtol = fmaxf((float)a.rtol, 2e-6f), jump_tol = 2e-5f;
+        for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.n; base += stride) {
+            const int64_t i = base + threadIdx.x;
+            if (i < a.n) {
+                const float hs = __ldg(a.hstar + i), p = __ldg(a.p + i), Tg = __ldg(a.Tg + i);
+                Comp<float, NS> c;
+                bool ok = load_comp<float, NS>(c, a.Y, a.ldY, i, a.N, s.sp);
+                ok = ok && isfinite(hs) && isfinite(Tg) && (p > 0.f) && isfinite(p);
+                int st = kBadInput, it = 0;
+                Temp2 Tres = {__int_as_float(0x7fc00000), 0.f};
+                if (ok) {
+                    const float T0 = fminf(fmaxf(Tg, (float)kTLo), (float)kTHi);
+                    float cp_last;
+                    st = newton_solve_f32<RZ, NS, KIJ>(c, hs, p, T0, s.sp, s.kij, (float)a.tmid_u, a.max_iter, rtol,
+                                                       jump_tol, Tres, it, cp_last);
+                    if constexpr (kMixed) {
+                        // FP64 where FP32 is least reliable: failed cells, and cells in
+                        // the pseudo-boiling band, from the FP32 root (or the guess)
+                        if (st != kOk || cp_last > (float)kPseudoCriticalCp * cp_ideal_mass<float, NS>(c, Tres.h, s.sp)) {
+                            const int e = atomicAdd(&q_n, 1);
+                            q_i[e] = i;
+                            q_h[e] = st == kOk ? Tres.h : T0;
+                            q_l[e] = st == kOk ? Tres.l : 0.f;
+                            q_it[e] = it;
+                        }
                     }
+                }
+                a.Tout[i] = Tres.h;
+                a.status[i] = st;
+                if (a.iters) a.iters[i] = it;
+            }
+            if constexpr (kMixed) {
+                __syncthreads();
+                while (q_n >= (int)blockDim.x) {
+                    finish(q_n - (int)blockDim.x + (int)threadIdx.x);
+                    __syncthreads();
+                    if (threadIdx.x == 0) q_n -= (int)blockDim.x;
+                    __syncthreads();
                 }
             }
         }
-        a.Tout[i] = (Real)Tres;
-        a.status[i] = st;
-        if (a.iters) a.iters[i] = it;
+        if (kMixed && (int)threadIdx.x < q_n) finish((int)threadIdx.x);
     }
 }
 
