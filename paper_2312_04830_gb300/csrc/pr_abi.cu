@@ -10,6 +10,7 @@
 #include <new>
 
 #include "pr_internal.h"
+#include "pr_fix9.cuh"
 #include "pr_kernels.cuh"
 
 using namespace prk;
@@ -132,6 +133,95 @@ void fill_occ(int NS, int occ_p[2], int occ_n[2])
 
 bool bad_double(double v) { return !std::isfinite(v); }
 
+typedef long double ld;   // at least 64 significant bits on x86-64 and aarch64
+
+// Values v[n] as fixed-point constants below 2^58 units of 2^e (e returned).
+int to_mac31(const ld *v, int n, Mac31 *const *out)
+{
+    ld top = 0;
+    for (int i = 0; i < n; ++i) top = fmaxl(top, fabsl(v[i]));
+    int e = 0;
+    if (top > 0) frexpl(top, &e);   // top < 2^e
+    e -= 58;
+    for (int i = 0; i < n; ++i) {
+        const int64_t q = (int64_t)roundl(ldexpl(v[i], -e));
+        out[i]->h = (int32_t)(q >> 31);
+        out[i]->l = (int32_t)(q & 0x7FFFFFFF);
+    }
+    return e;
+}
+
+// The fixed-point evaluation's tables (pr_fix9.cuh) of a context that takes
+// it; false otherwise.
+bool fill_fix9(Fix9 &t, const HostTable &h, int N, int flags, bool has_kij, double tmid_u)
+{
+    if (has_kij || N > 9 || !(tmid_u > 32.0 && tmid_u <= 1024.0)) return false;
+    memset(&t, 0, sizeof(t));
+    const ld Rg = kR;
+    const ld Oa = (flags & PR_FLAG_PRINTED_CONSTANTS) ? kOmegaAPrinted : kOmegaA;
+    const ld Ob = (flags & PR_FLAG_PRINTED_CONSTANTS) ? kOmegaBPrinted : kOmegaB;
+    memcpy(&t.Tmid, &tmid_u, 8);
+    ld iWmax = 0;
+    for (int k = 0; k < N; ++k) iWmax = fmaxl(iWmax, 1.0L / ((ld)h.W[k] * 1e-3L));
+    t.iWmax = (double)iWmax;
+    t.rWmax = (double)(1.0L / iWmax);
+    ld v[9] = {};
+    Mac31 *out[9] = {};
+    auto column = [&](Mac31 Fix9Rec::*f, auto value) {
+        for (int k = 0; k < N; ++k) {
+            v[k] = value(k);
+            out[k] = &(t.sp[k].*f);
+        }
+        return to_mac31(v, N, out);
+    };
+    ld kap[9], kq[9], g[9];
+    for (int k = 0; k < 9; ++k) {
+        const double inf = INFINITY;
+        memcpy(&t.sp[k].T0, &inf, 8);
+        if (k >= N) continue;
+        const ld r = roundl(ldexpl(1.0L / ((ld)h.W[k] * 1e-3L) / iWmax, 64));
+        t.sp[k].iW = r < 18446744073709551615.0L ? (uint64_t)r : ~0ull;
+        const ld w = h.omega[k];
+        kap[k] = 0.37464L + 1.54226L * w - 0.26992L * w * w;
+        kq[k] = kap[k] / sqrtl((ld)h.Tc[k]);
+        g[k] = sqrtl(Oa) * Rg * (ld)h.Tc[k] / sqrtl((ld)h.pc[k]);
+        if (!(1.0L + kap[k] > 0)) return false;
+        if (kq[k] > 0) {   // u_k changes sign once, at this temperature
+            const double T0 = (double)(((1.0L + kap[k]) / kq[k]) * ((1.0L + kap[k]) / kq[k]));
+            memcpy(&t.sp[k].T0, &T0, 8);
+        }
+    }
+    t.eb = column(&Fix9Rec::b, [&](int k) { return Ob * Rg * (ld)h.Tc[k] / (ld)h.pc[k]; });
+    t.eu0 = column(&Fix9Rec::u0, [&](int k) { return g[k] * (1.0L + kap[k]); });
+    t.eu1 = column(&Fix9Rec::u1, [&](int k) { return g[k] * kq[k]; });
+    // NASA-7: the five cp coefficients of a range in one unit, R a_6 of both in another
+    ld w5[45], w6[18];
+    Mac31 *o5[45], *o6[18];
+    for (int r = 0; r < 2; ++r) {
+        const ld scale = r ? 4096.0L : 1024.0L;
+        for (int k = 0; k < N; ++k) {
+            const double *a = r ? h.nasa_hi[k] : h.nasa_lo[k];
+            ld f = Rg;
+            for (int j = 0; j < 5; ++j, f *= scale) {
+                w5[5 * k + j] = f * (ld)a[j];
+                o5[5 * k + j] = &t.sp[k].nasa[r][j];
+            }
+            w6[9 * r + k] = Rg * (ld)a[5];
+            o6[9 * r + k] = &t.sp[k].nasa[r][5];
+        }
+        for (int k = N; k < 9; ++k) {
+            w6[9 * r + k] = 0;
+            o6[9 * r + k] = &t.sp[k].nasa[r][5];
+        }
+        t.en[r] = to_mac31(w5, 5 * N, o5);
+    }
+    t.ea6 = to_mac31(w6, 18, o6);
+    // every unit within a normal double's exponents
+    for (int e : {t.eb, t.eu0, t.eu1, t.en[0], t.en[1], t.ea6})
+        if (e < -800 || e > 800) return false;
+    return true;
+}
+
 }  // namespace
 
 // ===================================================================== ABI
@@ -225,6 +315,12 @@ pr_status pr_create(const pr_species_table *tbl, pr_ctx **out)
     c->tmid_u = h->T_mid[0] > 0 ? h->T_mid[0] : 0.0;
     for (int k = 1; k < N; ++k)
         if (h->T_mid[k] != h->T_mid[0]) c->tmid_u = 0.0;
+    if (e == cudaSuccess && NS == 9) {
+        Fix9 *f = new (std::nothrow) Fix9();
+        if (!f) e = cudaErrorMemoryAllocation;
+        else if (fill_fix9(*f, *h, N, c->flags, has_kij, c->tmid_u)) c->h_fix9 = f;
+        else delete f;
+    }
     if (d_tab) cudaFree(d_tab);
     delete h;
     if (e != cudaSuccess) {
@@ -236,6 +332,7 @@ pr_status pr_create(const pr_species_table *tbl, pr_ctx **out)
         pr_destroy(c);
         return ss;
     }
+    if (c->h_fix9) c->occ_fix = occupancy_newton_fix();
     fill_occ<double, double>(NS, c->occ_props[PR_FP64], c->occ_newton[PR_FP64]);
     fill_occ<float, float>(NS, c->occ_props[PR_FP32], c->occ_newton[PR_FP32]);
     fill_occ<float, double>(NS, c->occ_props[PR_MIXED], c->occ_newton[PR_MIXED]);
@@ -262,6 +359,7 @@ void pr_destroy(pr_ctx *c)
     prgb::species_tables_free(c);
     delete static_cast<HostTab9<double> *>(c->h_tab64);
     delete static_cast<HostTab9<float> *>(c->h_tab32);
+    delete static_cast<Fix9 *>(c->h_fix9);
     delete c;
 }
 
@@ -357,7 +455,9 @@ pr_status pr_T_from_h(pr_ctx *ctx, pr_precision prec, int64_t n, const void *hst
                              ctx->n_species, ctx->flags, max_iter, rtol,
                              (const SpeciesRec<float> *)ctx->d_sp32, ctx->d_pair32, ctx->d_kij32,
                              nullptr, nullptr, nullptr, ctx->tmid_u};
-        if (ctx->ns_pad == 9) launch_newton<double, double, 9>(a, kij, occ, ctx->num_sms, st);
+        if (ctx->h_fix9 && !(ctx->flags & PR_FLAG_NEWTON_FP64_ONLY))
+            launch_newton_fix(a, *static_cast<const Fix9 *>(ctx->h_fix9), ctx->occ_fix, ctx->num_sms, st);
+        else if (ctx->ns_pad == 9) launch_newton<double, double, 9>(a, kij, occ, ctx->num_sms, st);
         else launch_newton<double, double, 32>(a, kij, occ, ctx->num_sms, st);
     } else {
         NewtonArgs<float> a{n, ldY, (const float *)hstar, (const float *)p, (const float *)Y, (const float *)T_guess,

@@ -74,6 +74,10 @@ struct pr_ctx {
     // the property kernels take by value; NULL for the 32-species kernels
     void *h_tab64;
     void *h_tab32;
+    // tables of the fixed-point FP64 kernels (pr_fix9.cuh), or NULL when the
+    // context does not take them; the inversion kernel's resident blocks per SM
+    void *h_fix9;
+    int occ_fix;
     double tmid_u;       // common NASA-7 switch temperature of every species, or 0
     // device address of the allocation-free entry point's scratch array on
     // this context's device (noalloc.cu), or NULL if the lookup failed

@@ -292,17 +292,12 @@ __device__ __noinline__ int eval_h_f32(const Comp<float, NS> &c, float T, float 
 // conversion.  cp_end: the FP32 cp at the returned root (0 if that
 // evaluation fails), for the first FP64 step.
 template <int NS, bool KIJ>
-__device__ __noinline__ double warm_start_fp32(const Comp<double, NS> &c64, double T0, double hs, double p,
+__device__ __noinline__ double warm_start_fp32(const Comp<float, NS> &c, double T0, double hs, double p,
                                                const SpeciesRec<float> *sp, const float *kij, float tmid_u, bool &ok,
                                                float &cp_end)
 {
     ok = false;
     cp_end = 0.f;
-    Comp<float, NS> c;
-#pragma unroll
-    for (int k = 0; k < NS; ++k) c.x[k] = (float)c64.x[k];
-    c.Wbar = (float)c64.Wbar;
-    c.bm = (float)c64.bm;
     const float hsf = (float)hs, pf = (float)p;
     float T = (float)T0;
 #pragma unroll 1
@@ -550,7 +545,12 @@ __device__ __forceinline__ void newton_fp64_queued(const NewtonArgs<double> &a, 
             } else {
                 bool wok;
                 float cp32;
-                const double T = warm_start_fp32<NS, KIJ>(c, fmin(fmax(Tg, kTLo), kTHi), hs, p, s32.sp, s32.kij,
+                Comp<float, NS> c32;
+#pragma unroll
+                for (int k = 0; k < NS; ++k) c32.x[k] = (float)c.x[k];
+                c32.Wbar = (float)c.Wbar;
+                c32.bm = (float)c.bm;
+                const double T = warm_start_fp32<NS, KIJ>(c32, fmin(fmax(Tg, kTLo), kTHi), hs, p, s32.sp, s32.kij,
                                                           (float)a.tmid_u, wok, cp32);
                 bool accepted = false, first = false;
                 double h0 = 0.0, cp0 = 0.0;
