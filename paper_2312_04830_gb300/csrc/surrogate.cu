@@ -778,18 +778,19 @@ EncodeTiledFn encode_fn()
 }
 
 // K-major BF16 operand [rows][inner] with row pitch `pitch` elements, loaded
-// in boxes of 64 x box_rows with 128-byte swizzling (out-of-range rows and
-// columns read as zero).
-bool make_map(CUtensorMap *m, const void *ptr, uint64_t inner, uint64_t rows, uint64_t pitch, uint32_t box_rows)
+// in boxes of 64 x box_rows with 128-byte swizzling, or of 32 x box_rows with
+// 64-byte swizzling (out-of-range rows and columns read as zero).
+bool make_map(CUtensorMap *m, const void *ptr, uint64_t inner, uint64_t rows, uint64_t pitch, uint32_t box_rows,
+              uint32_t box_cols = 64)
 {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[2] = {inner, rows};
     cuuint64_t strides[1] = {pitch * 2};
-    cuuint32_t box[2] = {64, box_rows};
+    cuuint32_t box[2] = {box_cols, box_rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, box_cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
@@ -953,15 +954,12 @@ void fused_lag(int G, int ips, int &D, int &ring)
     ring = 2 * D + 4;
 }
 
-// The resident-activation kernel for width W (256 or 512) and this depth (the
-// output layer's weights resident in shared memory when they fit).
+// The resident-activation kernel for width W (256 or 512) and this depth.
 inline const void *resident_fn(int L, int W)
 {
-    const bool wo = ResCfg::wout_resident(L, W);
-    if (W == 256) return wo ? reinterpret_cast<const void *>(mlp_resident_kernel<256, true>)
-                            : reinterpret_cast<const void *>(mlp_resident_kernel<256, false>);
-    return wo ? reinterpret_cast<const void *>(mlp_resident_kernel<512, true>)
-              : reinterpret_cast<const void *>(mlp_resident_kernel<512, false>);
+    if (ResCfg::stages(L, W) == 3) return reinterpret_cast<const void *>(mlp_resident_kernel<512, 3>);
+    return W == 256 ? reinterpret_cast<const void *>(mlp_resident_kernel<256, 4>)
+                    : reinterpret_cast<const void *>(mlp_resident_kernel<512, 4>);
 }
 
 // CTA pairs of the resident-activation kernel the device holds at once (0:
@@ -981,7 +979,7 @@ int resident_pairs(int L, int W)
     attr[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(2 * num_sms_current(), 1, 1);
     cfg.blockDim = dim3(kResThreads, 1, 1);
-    cfg.dynamicSmemBytes = ResCfg::smem_bytes(L, W, ResCfg::wout_resident(L, W));
+    cfg.dynamicSmemBytes = ResCfg::smem_bytes(L, W, ResCfg::stages(L, W));
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int nc = 0;
@@ -1061,7 +1059,6 @@ cudaError_t launch_resident(const ResidentArgs &ra, int pairs, cudaStream_t st)
 {
     const int R = (ra.M + 255) / 256;
     const int g = R < pairs ? R : pairs;
-    const bool wo = ResCfg::wout_resident(ra.L, ra.W);
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1070,15 +1067,13 @@ cudaError_t launch_resident(const ResidentArgs &ra, int pairs, cudaStream_t st)
     attr[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3((unsigned)(2 * g), 1, 1);
     cfg.blockDim = dim3(kResThreads, 1, 1);
-    cfg.dynamicSmemBytes = ResCfg::smem_bytes(ra.L, ra.W, wo);
+    cfg.dynamicSmemBytes = ResCfg::smem_bytes(ra.L, ra.W, ResCfg::stages(ra.L, ra.W));
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (ra.W == 256)
-        return wo ? cudaLaunchKernelEx(&cfg, mlp_resident_kernel<256, true>, ra)
-                  : cudaLaunchKernelEx(&cfg, mlp_resident_kernel<256, false>, ra);
-    return wo ? cudaLaunchKernelEx(&cfg, mlp_resident_kernel<512, true>, ra)
-              : cudaLaunchKernelEx(&cfg, mlp_resident_kernel<512, false>, ra);
+    if (ResCfg::stages(ra.L, ra.W) == 3) return cudaLaunchKernelEx(&cfg, mlp_resident_kernel<512, 3>, ra);
+    return ra.W == 256 ? cudaLaunchKernelEx(&cfg, mlp_resident_kernel<256, 4>, ra)
+                       : cudaLaunchKernelEx(&cfg, mlp_resident_kernel<512, 4>, ra);
 }
 
 GemmArgs base_args(sg_model *m)
@@ -1143,6 +1138,7 @@ static pr_status build_maps(sg_model *m)
             ok = ok && make_map(&m->tmr_w[0], d.wb[0], KIN, W, KIN, (uint32_t)(W / 4));
             for (int l = 1; l < L; ++l) ok = ok && make_map(&m->tmr_w[l], d.wb[l], W, W, W, (uint32_t)(W / 4));
             ok = ok && make_map(&m->tmr_w[L], d.wb[L], W, NOP, W, 8);
+            ok = ok && make_map(&m->tmr_x, d.xi, KIN, C, KIN, 128, kResXCols);
         }
         if (m->pp_pairs > 0) {   // alternating activations: a CTA's 64 rows of every 128-row N-tile
             ok = ok && make_map(&m->tmq_w[0], d.wb[0], KIN, W, KIN, (uint32_t)(kPPBN / 2));
@@ -1559,7 +1555,7 @@ pr_status surrogate_infer(sg_model *m, int64_t n, const float *T, const float *p
             const bool pp = m->fused_on == 4;
             ResidentArgs ra;
             memset(&ra, 0, sizeof(ra));
-            ra.tm_x = m->tm_xi;
+            ra.tm_x = pp ? m->tm_xi : m->tmr_x;
             for (int l = 0; l <= L; ++l) {
                 ra.tm_w[l] = pp ? m->tmq_w[l] : m->tmr_w[l];
                 ra.bias[l] = d.master + d.lay[l].b_off;

@@ -128,9 +128,10 @@ struct sg_model {
     CUtensorMap tmf_w[SG_MAX_HIDDEN + 1], tmf_ring_ld, tmf_ring_st;
     CUtensorMap tmp_w[SG_MAX_HIDDEN + 1];  // CTA pairs: half-height weight boxes
     // resident-activation inference (mlp_resident.cuh): CTA pairs held at
-    // once (0: not available for this shape), weight boxes of W / 4 rows
+    // once (0: not available for this shape), weight boxes of W / 4 rows,
+    // input boxes of 32 columns
     int res_pairs;
-    CUtensorMap tmr_w[SG_MAX_HIDDEN + 1];
+    CUtensorMap tmr_w[SG_MAX_HIDDEN + 1], tmr_x;
     // activations alternating between tensor and shared memory
     // (mlp_pingpong.cuh): CTA pairs the device holds at once, and the weight
     // maps (boxes of 64 rows: a CTA's half of a 128-row N-tile)

@@ -393,6 +393,19 @@ __device__ __forceinline__ uint64_t sdesc_kmajor_sw128(uint32_t saddr)
     return d;
 }
 
+// The same for rows of 32 BF16 (64 B) with 64-byte swizzling: 8-row atoms of
+// 512 B (stride offset 512 B), swizzle mode 4.
+__device__ __forceinline__ uint64_t sdesc_kmajor_sw64(uint32_t saddr)
+{
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(16u >> 4) << 16;
+    d |= (uint64_t)(512u >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)4 << 61;
+    return d;
+}
+
 // Shared-memory matrix descriptor of an MN-major operand tile written by TMA
 // with 128-byte swizzling: each 128-byte row holds 64 consecutive M (or N)
 // elements of one k, and rows of consecutive k follow one another, so 8-row
