@@ -332,7 +332,7 @@ pr_status pr_create(const pr_species_table *tbl, pr_ctx **out)
         pr_destroy(c);
         return ss;
     }
-    if (c->h_fix9) c->occ_fix = occupancy_newton_fix();
+    if (c->h_fix9) occupancy_newton_fix(c->occ_fix);
     fill_occ<double, double>(NS, c->occ_props[PR_FP64], c->occ_newton[PR_FP64]);
     fill_occ<float, float>(NS, c->occ_props[PR_FP32], c->occ_newton[PR_FP32]);
     fill_occ<float, double>(NS, c->occ_props[PR_MIXED], c->occ_newton[PR_MIXED]);
@@ -456,7 +456,7 @@ pr_status pr_T_from_h(pr_ctx *ctx, pr_precision prec, int64_t n, const void *hst
                              (const SpeciesRec<float> *)ctx->d_sp32, ctx->d_pair32, ctx->d_kij32,
                              nullptr, nullptr, nullptr, ctx->tmid_u};
         if (ctx->h_fix9 && !(ctx->flags & PR_FLAG_NEWTON_FP64_ONLY))
-            launch_newton_fix(a, *static_cast<const Fix9 *>(ctx->h_fix9), ctx->occ_fix, ctx->num_sms, st);
+            launch_newton_fix(a, *static_cast<const Fix9 *>(ctx->h_fix9), ctx->h_tab32, ctx->occ_fix, ctx->num_sms, st);
         else if (ctx->ns_pad == 9) launch_newton<double, double, 9>(a, kij, occ, ctx->num_sms, st);
         else launch_newton<double, double, 32>(a, kij, occ, ctx->num_sms, st);
     } else {

@@ -20,13 +20,114 @@ static __device__ __noinline__ void newton_finish9(const NewtonArgs<double> &a, 
     if (a.iters) a.iters[i] = it;
 }
 
-// newton_fp64_queued (pr_kernels.cuh) with the first FP64 evaluation in fixed
-// point; the FP32 warm start takes its mole fractions from the same limbs.
-// 2.1 M cells of the flame field: 1643 -> 1155 us (345 -> 126 FP64-pipe
-// instructions per cell, the pipe 74 -> 39 % busy; what holds it now is
-// instruction fetch, 4.4 of 9 stall cycles per issue).
+// The inversion in two launches: in one kernel the FP32 iterations and the
+// FP64 evaluation missed the instruction cache (half of the stall cycles) and
+// ran at the FP64 part's 128 registers.  First the FP32 warm start of every cell, T
+// into Tout and the FP32 cp at it, as bits, into the status array (0 where
+// the warm start failed: T is then the clamped guess; -1: a guess refused) ...
+__global__ void __launch_bounds__(kBlock) newton_warm_kernel(const __grid_constant__ NewtonArgs<double> a,
+                                                             const __grid_constant__ ParamTab<float, 9, false> t)
+{
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += stride) {
+        const float hs = (float)__ldg(a.hstar + i), p = (float)__ldg(a.p + i);
+        const double Tg = a.Tg[i];   // Tg may be Tout
+        const double T0 = fmin(fmax(Tg, kTLo), kTHi);
+        Comp<float, 9> c;
+        float s = 0.f, bm = 0.f;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            c.x[k] = (k < a.N) ? (float)__ldg(a.Y + (int64_t)k * a.ldY + i) * t.sp[k].inv_W : 0.f;
+            s += c.x[k];
+        }
+        const float is = 1.f / s;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            c.x[k] *= is;
+            bm = fmaf(c.x[k], t.sp[k].b, bm);
+        }
+        c.Wbar = is;
+        c.bm = bm;
+        // warm_start_fp32's iteration with its evaluations at one place, in
+        // line, the tables as constant operands (states refused by the second
+        // launch pass through here too: the loop is bounded)
+        float T = (float)T0, cp_end = 0.f;
+        bool ok = false;
+#pragma unroll 1
+        for (int k = 0; k < 9; ++k) {
+            Thermo<float> th;
+            thermo<float, float, 9, false>(c, T, p, t.sp, t.kij, th, (float)a.tmid_u);
+            if (th.status == kNoRoot || !(th.cp > 0.f)) break;
+            if (ok) {   // the step before was the last one: cp at the root
+                cp_end = th.cp;
+                break;
+            }
+            const float Tn = T - (th.h - hs) / th.cp;
+            if (!(Tn > (float)kTLo && Tn < (float)kTHi) || k == 8) break;
+            ok = fabsf(Tn - T) <= 1e-5f * Tn;
+            T = Tn;
+        }
+        a.Tout[i] = cp_end > 0.f ? (double)T : T0;
+        a.status[i] = __float_as_int(isfinite(Tg) ? cp_end : -1.f);
+    }
+}
+
+// ... then one FP64 evaluation per cell, in fixed point, and the one-step
+// acceptance; the other cells through a queue of the block, as
+// newton_fp64_queued (pr_kernels.cuh).
+__device__ __forceinline__ void newton_fix_cell(const NewtonArgs<double> &a, const Fix9 &t, int64_t i, double T,
+                                                float cp32, const SpeciesRec<float> *sp32, int *q_n,
+                                                int64_t *q_i, double *q_T, double *q_h, double *q_cp,
+                                                unsigned char *q_first, bool guess_ok)
+{
+    const double hs = __ldg(a.hstar + i), p = __ldg(a.p + i);
+    double y[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) y[k] = (k < a.N) ? __ldg(a.Y + (int64_t)k * a.ldY + i) : 0.0;
+    Fix9Comp c;
+    const int ok = fix9_comp(t, y, c);
+    if (ok == kFixBad || !(guess_ok && isfinite(hs) && p > 0.0 && isfinite(p))) {
+        a.Tout[i] = M<double>::nan();
+        a.status[i] = kBadInput;
+        if (a.iters) a.iters[i] = 0;
+        return;
+    }
+    bool first = false;
+    double h0 = 0.0, cp0 = 0.0;
+    if (ok == kFixOk && cp32 > 0.f && fix9_range(T)) {
+        Thermo<double> th;
+        fix9_thermo(t, c, T, p, th);
+        if (th.status != kNoRoot) {
+            FirstEval f;
+            f.status = th.status;
+            f.nroots = th.nroots;
+            f.h = th.h;
+            f.cp = (double)cp32;
+            f.cv_ig = (float)th.cv_ig_molar;
+            const double dT = m64::div(hs - f.h, f.cp);
+            if (one_step_ok<9>(f, T, dT, c.Wbar, sp32, (float)a.tmid_u)) {
+                a.Tout[i] = T + dT;
+                a.status[i] = kOk;
+                if (a.iters) a.iters[i] = 1;
+                return;
+            }
+            first = true;
+            h0 = f.h;
+            cp0 = f.cp;
+        }
+    }
+    const int e = atomicAdd(q_n, 1);
+    q_i[e] = i;
+    q_T[e] = T;
+    q_h[e] = h0;
+    q_cp[e] = cp0;
+    q_first[e] = first ? 1 : 0;
+}
+
+// SPLIT: T and cp from newton_warm_kernel; else the warm start runs here.
+template <bool SPLIT>
 __global__ void __launch_bounds__(kBlock, 4) newton_fix_kernel(const __grid_constant__ NewtonArgs<double> a,
-                                                            const __grid_constant__ Fix9 t)
+                                                               const __grid_constant__ Fix9 t)
 {
     __shared__ Smem<float, 9, false> s32;
     __shared__ int q_n;
@@ -39,65 +140,31 @@ __global__ void __launch_bounds__(kBlock, 4) newton_fix_kernel(const __grid_cons
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.n; base += stride) {
         const int64_t i = base + threadIdx.x;
         if (i < a.n) {
-            const double hs = __ldg(a.hstar + i), p = __ldg(a.p + i), Tg = __ldg(a.Tg + i);
-            double y[9];
-#pragma unroll
-            for (int k = 0; k < 9; ++k) y[k] = (k < a.N) ? __ldg(a.Y + (int64_t)k * a.ldY + i) : 0.0;
-            Fix9Comp c;
-            const int ok = fix9_comp(t, y, c);
-            if (ok == kFixBad || !(isfinite(hs) && isfinite(Tg) && p > 0.0 && isfinite(p))) {
-                a.Tout[i] = M<double>::nan();
-                a.status[i] = kBadInput;
-                if (a.iters) a.iters[i] = 0;
+            if constexpr (SPLIT) {
+                const float cp32 = __int_as_float(a.status[i]);
+                newton_fix_cell(a, t, i, a.Tout[i], cp32, s32.sp, &q_n, q_i, q_T, q_h, q_cp, q_first, cp32 >= 0.f);
             } else {
-                double T = fmin(fmax(Tg, kTLo), kTHi);
-                bool accepted = false, first = false;
-                double h0 = 0.0, cp0 = 0.0;
-                if (ok == kFixOk) {
-                    Comp<float, 9> cf;
-                    float bm = 0.f;
+                const double Tg = __ldg(a.Tg + i);
+                Comp<float, 9> cf;
+                float s = 0.f, bm = 0.f;
 #pragma unroll
-                    for (int k = 0; k < 9; ++k) {
-                        cf.x[k] = (float)c.xh[k] * 4.6566128730773926e-10f;   // 2^-31
-                        bm = fmaf(cf.x[k], s32.sp[k].b, bm);
-                    }
-                    cf.Wbar = (float)c.Wbar;
-                    cf.bm = bm;
-                    bool wok;
-                    float cp32;
-                    T = warm_start_fp32<9, false>(cf, T, hs, p, s32.sp, s32.kij, (float)a.tmid_u, wok, cp32);
-                    if (wok && cp32 > 0.f && fix9_range(T)) {
-                        Thermo<double> th;
-                        fix9_thermo(t, c, T, p, th);
-                        if (th.status != kNoRoot) {
-                            FirstEval f;
-                            f.status = th.status;
-                            f.nroots = th.nroots;
-                            f.h = th.h;
-                            f.cp = (double)cp32;
-                            f.cv_ig = (float)th.cv_ig_molar;
-                            const double dT = m64::div(hs - f.h, f.cp);
-                            if (one_step_ok<9>(f, T, dT, c.Wbar, s32.sp, (float)a.tmid_u)) {
-                                a.Tout[i] = T + dT;
-                                a.status[i] = kOk;
-                                if (a.iters) a.iters[i] = 1;
-                                accepted = true;
-                            } else {
-                                first = true;
-                                h0 = f.h;
-                                cp0 = f.cp;
-                            }
-                        }
-                    }
+                for (int k = 0; k < 9; ++k) {
+                    cf.x[k] = (k < a.N) ? (float)__ldg(a.Y + (int64_t)k * a.ldY + i) * s32.sp[k].inv_W : 0.f;
+                    s += cf.x[k];
                 }
-                if (!accepted) {
-                    const int e = atomicAdd(&q_n, 1);
-                    q_i[e] = i;
-                    q_T[e] = T;
-                    q_h[e] = h0;
-                    q_cp[e] = cp0;
-                    q_first[e] = first ? 1 : 0;
+                const float is = 1.f / s;
+#pragma unroll
+                for (int k = 0; k < 9; ++k) {
+                    cf.x[k] *= is;
+                    bm = fmaf(cf.x[k], s32.sp[k].b, bm);
                 }
+                cf.Wbar = is;
+                cf.bm = bm;
+                bool wok;
+                float cp32;
+                const double T = warm_start_fp32<9, false>(cf, fmin(fmax(Tg, kTLo), kTHi), __ldg(a.hstar + i),
+                                                           __ldg(a.p + i), s32.sp, s32.kij, (float)a.tmid_u, wok, cp32);
+                newton_fix_cell(a, t, i, T, wok ? cp32 : 0.f, s32.sp, &q_n, q_i, q_T, q_h, q_cp, q_first, isfinite(Tg));
             }
         }
         __syncthreads();
@@ -115,16 +182,41 @@ __global__ void __launch_bounds__(kBlock, 4) newton_fix_kernel(const __grid_cons
     }
 }
 
-void launch_newton_fix(const NewtonArgs<double> &a, const Fix9 &t, int occ, int sms, cudaStream_t st)
+// [a, a + na) and [b, b + nb) share a byte
+static bool overlap(const void *a, size_t na, const void *b, size_t nb)
 {
-    newton_fix_kernel<<<grid_for(a.n, occ, sms), kBlock, 0, st>>>(a, t);
+    const char *x = static_cast<const char *>(a), *y = static_cast<const char *>(b);
+    return x < y + nb && y < x + na;
 }
 
-int occupancy_newton_fix()
+void launch_newton_fix(const NewtonArgs<double> &a, const Fix9 &t, const void *htab32, const int occ[3], int sms,
+                       cudaStream_t st)
 {
-    int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, newton_fix_kernel, kBlock, 0);
-    return occ > 0 ? occ : 1;
+    // the first launch writes Tout and status: only the guess may be among
+    // them (element by element), not what the second launch reads
+    const size_t nb = (size_t)a.n * 8, yb = ((size_t)a.ldY * (size_t)(a.N - 1) + (size_t)a.n) * 8;
+    const bool own = !overlap(a.Tout, nb, a.hstar, nb) && !overlap(a.Tout, nb, a.p, nb) && !overlap(a.Tout, nb, a.Y, yb) &&
+                     (a.Tout == a.Tg || !overlap(a.Tout, nb, a.Tg, nb)) && !overlap(a.status, nb / 2, a.Tout, nb) &&
+                     !overlap(a.status, nb / 2, a.hstar, nb) && !overlap(a.status, nb / 2, a.p, nb) &&
+                     !overlap(a.status, nb / 2, a.Y, yb) && !overlap(a.status, nb / 2, a.Tg, nb);
+    // two launches for more cells than one wave of the single kernel holds:
+    // up to there the second launch costs more than the smaller kernels gain
+    // (65536 cells, in one wave: 69 us against 72; 131072: 114 against 88;
+    // 2.1 M cells: 1238 against 683)
+    if (a.n > (int64_t)occ[2] * sms * kBlock && own) {
+        newton_warm_kernel<<<grid_for(a.n, occ[0], sms), kBlock, 0, st>>>(a, make_tab<float, 9, false>(htab32));
+        newton_fix_kernel<true><<<grid_for(a.n, occ[1], sms), kBlock, 0, st>>>(a, t);
+    } else {
+        newton_fix_kernel<false><<<grid_for(a.n, occ[2], sms), kBlock, 0, st>>>(a, t);
+    }
+}
+
+void occupancy_newton_fix(int occ[3])
+{
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[0], newton_warm_kernel, kBlock, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[1], newton_fix_kernel<true>, kBlock, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[2], newton_fix_kernel<false>, kBlock, 0);
+    for (int k = 0; k < 3; ++k) occ[k] = occ[k] > 0 ? occ[k] : 1;
 }
 
 }  // namespace prk

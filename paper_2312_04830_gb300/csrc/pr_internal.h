@@ -75,9 +75,9 @@ struct pr_ctx {
     void *h_tab64;
     void *h_tab32;
     // tables of the fixed-point FP64 kernels (pr_fix9.cuh), or NULL when the
-    // context does not take them; the inversion kernel's resident blocks per SM
+    // context does not take them; the inversion kernels' resident blocks per SM
     void *h_fix9;
-    int occ_fix;
+    int occ_fix[3];
     double tmid_u;       // common NASA-7 switch temperature of every species, or 0
     // device address of the allocation-free entry point's scratch array on
     // this context's device (noalloc.cu), or NULL if the lookup failed
