@@ -457,8 +457,8 @@ pr_status pr_T_from_h(pr_ctx *ctx, pr_precision prec, int64_t n, const void *hst
                              nullptr, nullptr, nullptr, ctx->tmid_u};
         if (ctx->h_fix9 && !(ctx->flags & PR_FLAG_NEWTON_FP64_ONLY))
             launch_newton_fix(a, *static_cast<const Fix9 *>(ctx->h_fix9), ctx->h_tab32, ctx->occ_fix, ctx->num_sms, st);
-        else if (ctx->ns_pad == 9) launch_newton<double, double, 9>(a, kij, occ, ctx->num_sms, st);
-        else launch_newton<double, double, 32>(a, kij, occ, ctx->num_sms, st);
+        else if (ctx->ns_pad == 9) launch_newton<double, double, 9>(a, nullptr, kij, occ, ctx->num_sms, st);
+        else launch_newton<double, double, 32>(a, nullptr, kij, occ, ctx->num_sms, st);
     } else {
         NewtonArgs<float> a{n, ldY, (const float *)hstar, (const float *)p, (const float *)Y, (const float *)T_guess,
                             (float *)T_out, cell_status, iters, (const SpeciesRec<float> *)ctx->d_sp32,
@@ -466,11 +466,11 @@ pr_status pr_T_from_h(pr_ctx *ctx, pr_precision prec, int64_t n, const void *hst
                             nullptr, nullptr, nullptr,
                             (const SpeciesRec<double> *)ctx->d_sp64, ctx->d_pair64, ctx->d_kij64, ctx->tmid_u};
         if (prec == PR_FP32) {
-            if (ctx->ns_pad == 9) launch_newton<float, float, 9>(a, kij, occ, ctx->num_sms, st);
-            else launch_newton<float, float, 32>(a, kij, occ, ctx->num_sms, st);
+            if (ctx->ns_pad == 9) launch_newton<float, float, 9>(a, ctx->h_tab32, kij, occ, ctx->num_sms, st);
+            else launch_newton<float, float, 32>(a, nullptr, kij, occ, ctx->num_sms, st);
         } else {
-            if (ctx->ns_pad == 9) launch_newton<float, double, 9>(a, kij, occ, ctx->num_sms, st);
-            else launch_newton<float, double, 32>(a, kij, occ, ctx->num_sms, st);
+            if (ctx->ns_pad == 9) launch_newton<float, double, 9>(a, ctx->h_tab32, kij, occ, ctx->num_sms, st);
+            else launch_newton<float, double, 32>(a, nullptr, kij, occ, ctx->num_sms, st);
         }
     }
     PR_CUDA_TRY(cudaGetLastError());

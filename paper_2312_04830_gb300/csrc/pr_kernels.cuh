@@ -269,14 +269,13 @@ __device__ __forceinline__ bool one_step_ok(const FirstEval &f, double T, double
     return clear;
 }
 
-// h(T) and cp(T) in FP32 with FP32 arguments (the warm start's evaluations,
-// and the FP32 and mixed inversions').
-template <int NS, bool KIJ, typename RZ = float>
+// h(T) and cp(T) in FP32 with FP32 arguments (the warm start's evaluations).
+template <int NS, bool KIJ>
 __device__ __noinline__ int eval_h_f32(const Comp<float, NS> &c, float T, float p, const SpeciesRec<float> *sp,
                                        const float *kij, float tmid_u, float &h, float &cp)
 {
     Thermo<float> th;
-    thermo<float, RZ, NS, KIJ>(c, T, p, sp, kij, th, tmid_u);
+    thermo<float, float, NS, KIJ>(c, T, p, sp, kij, th, tmid_u);
     if (th.status == kNoRoot) return kNoRoot;
     h = th.h;
     cp = th.cp;
@@ -395,7 +394,9 @@ __device__ __forceinline__ bool temp2_less(Temp2 a, Temp2 b) { return a.h < b.h 
 // the tests in FP32.  In double, these ~25 FP64-pipe operations per iteration
 // (77 per cell) held the FP32 kernel, the pipe 80 % busy and the issue slots
 // 44 %: 4.5 M cells of the flame field 703 us (535 us with the division on
-// the integer pipe), 365 us with this bookkeeping, errors unchanged.
+// the integer pipe), 365 us with this bookkeeping, and 326 us with the
+// thermodynamics in line at one place and the tables in the parameter space
+// (35.5 M of 336 M instructions were loads of tables and arguments).
 template <typename RZ, int NS, bool KIJ>
 __device__ __forceinline__ int newton_solve_f32(const Comp<float, NS> &c, float hs, float p, float T0,
                                                 const SpeciesRec<float> *sp, const float *kij, float tmid_u,
@@ -403,48 +404,60 @@ __device__ __forceinline__ int newton_solve_f32(const Comp<float, NS> &c, float 
                                                 float &cp_last)
 {
     const float tlo = (float)kTLo, thi = (float)kTHi;
-    Temp2 lo = {tlo, 0.f}, hi = {thi, 0.f}, t = {T0, 0.f};
+    Temp2 lo = {tlo, 0.f}, hi = {thi, 0.f}, t = {T0, 0.f}, tn = t;
     bool lo_done = false, hi_done = false;   // endpoint h evaluated (range checked)
-    float fprev = INFINITY;
-    int st = kMaxIt, it;
+    float fprev = INFINITY, f = 0.f, Te = T0;
+    int st = kMaxIt, it = 1;
     Tres = t;
     cp_last = 0.f;
+    // the thermodynamics at one place, in line: at T (0), at a bracket end
+    // before leaning on it (1), at the last step's T (2)
+    int phase = 0;
 #pragma unroll 1
-    for (it = 1; it <= max_iter; ++it) {
-        float h, cp;
-        const int e = eval_h_f32<NS, KIJ, RZ>(c, t.h, p, sp, kij, tmid_u, h, cp);
-        if (e) { st = e; Tres = t; break; }
-        cp_last = cp;
-        const float f = h - hs;
-        if (fabsf(f) <= rtol * fmaxf(fabsf(hs), fabsf(cp) * t.h)) { st = kOk; Tres = t; break; }
-        if (f < 0) lo = t; else hi = t;
-        Temp2 tn = temp2_add(t, -(f / cp));
-        const bool newton_ok = (cp > 0) && temp2_less(lo, tn) && temp2_less(tn, hi) && (fabsf(f) <= 0.5f * fabsf(fprev));
-        if (!newton_ok) {
-            tn = temp2_add(temp2_add(lo, hi.h), hi.l);
-            tn.h *= 0.5f;
-            tn.l *= 0.5f;
-            if ((lo.h == tlo && lo.l == 0.f && !lo_done) || (hi.h == thi && hi.l == 0.f && !hi_done)) {
-                const bool use_lo = (lo.h == tlo && lo.l == 0.f && !lo_done);
-                const float Te = use_lo ? tlo : thi;
-                float he, cpe;
-                const int e2 = eval_h_f32<NS, KIJ, RZ>(c, Te, p, sp, kij, tmid_u, he, cpe);
-                if (e2) { st = e2; Tres = t; break; }
-                if (use_lo) lo_done = true; else hi_done = true;
-                if ((use_lo && hs < he) || (!use_lo && hs > he)) { st = kHRange; Tres = {Te, 0.f}; break; }
-            }
-        }
-        fprev = f;
-        if (fabsf((tn.h - t.h) + (tn.l - t.l)) <= rtol * t.h) {
-            Tres = tn;
-            float h2, cp2;
-            if (eval_h_f32<NS, KIJ, RZ>(c, tn.h, p, sp, kij, tmid_u, h2, cp2)) { st = kNoRoot; break; }
-            cp_last = cp2;
-            st = (fabsf(h2 - hs) <= jump_tol * fmaxf(fabsf(hs), fabsf(cp2) * tn.h)) ? kOk : kHRange;
+    while (true) {
+        Thermo<float> th;
+        thermo<float, RZ, NS, KIJ>(c, Te, p, sp, kij, th, tmid_u);
+        const float h = th.h, cp = th.cp;
+        if (phase == 2) {
+            if (th.status == kNoRoot) { st = kNoRoot; break; }
+            cp_last = cp;
+            st = (fabsf(h - hs) <= jump_tol * fmaxf(fabsf(hs), fabsf(cp) * tn.h)) ? kOk : kHRange;
             break;
         }
-        t = tn;
+        if (th.status == kNoRoot) { st = kNoRoot; Tres = t; break; }
+        if (phase == 0) {
+            cp_last = cp;
+            f = h - hs;
+            if (fabsf(f) <= rtol * fmaxf(fabsf(hs), fabsf(cp) * t.h)) { st = kOk; Tres = t; break; }
+            if (f < 0) lo = t; else hi = t;
+            tn = temp2_add(t, -(f / cp));
+            const bool newton_ok = (cp > 0) && temp2_less(lo, tn) && temp2_less(tn, hi) && (fabsf(f) <= 0.5f * fabsf(fprev));
+            if (!newton_ok) {
+                tn = temp2_add(temp2_add(lo, hi.h), hi.l);
+                tn.h *= 0.5f;
+                tn.l *= 0.5f;
+                const bool use_lo = lo.h == tlo && lo.l == 0.f && !lo_done;
+                if (use_lo || (hi.h == thi && hi.l == 0.f && !hi_done)) {
+                    Te = use_lo ? tlo : thi;
+                    phase = 1;
+                    continue;
+                }
+            }
+        } else {
+            const bool use_lo = Te == tlo;
+            if (use_lo) lo_done = true; else hi_done = true;
+            if ((use_lo && hs < h) || (!use_lo && hs > h)) { st = kHRange; Tres = {Te, 0.f}; break; }
+        }
+        fprev = f;
         Tres = tn;
+        Te = tn.h;
+        if (fabsf((tn.h - t.h) + (tn.l - t.l)) <= rtol * t.h) {
+            phase = 2;
+            continue;
+        }
+        phase = 0;
+        t = tn;
+        if (++it > max_iter) break;
     }
     iters = it > max_iter ? max_iter : it;
     return st;
@@ -592,16 +605,33 @@ __device__ __forceinline__ void newton_fp64_queued(const NewtonArgs<double> &a, 
     if ((int)threadIdx.x < q_n) finish((int)threadIdx.x);
 }
 
+// The FP32 and mixed kernels of up to 9 species take their FP32 tables in the
+// parameter space, as the property kernels do.
+template <typename Real, int NS, bool KIJ>
+using NewtonTab = typename std::conditional<NS == 9 && sizeof(Real) == 4, ParamTab<float, 9, KIJ>, NoTab>::type;
+
 template <typename Real, typename RZ, int NS, bool KIJ>
-__global__ void __launch_bounds__(kBlock) newton_kernel(const NewtonArgs<Real> a)
+__global__ void __launch_bounds__(kBlock) newton_kernel(const __grid_constant__ NewtonArgs<Real> a,
+                                                        const __grid_constant__ NewtonTab<Real, NS, KIJ> tab)
 {
-    __shared__ Smem<Real, NS, KIJ> s;
-    stage<Real, NS, KIJ>(s, a.sp, a.pair, a.kij);
+    constexpr bool kParam = NS == 9 && sizeof(Real) == 4;
+    __shared__ typename std::conditional<kParam, char, Smem<Real, NS, KIJ>>::type s_[1];
+    const SpeciesRec<Real> *sp;
+    const Real *kij;
+    if constexpr (kParam) {
+        sp = tab.sp;
+        kij = tab.kij;
+    } else {
+        stage<Real, NS, KIJ>(s_[0], a.sp, a.pair, a.kij);
+        sp = s_[0].sp;
+        kij = s_[0].kij;
+    }
     // FP64 inversion: FP32 tables for the warm start
     constexpr bool kFp64 = sizeof(Real) == 8;
-    __shared__ Smem<float, NS, KIJ> s32[1];
+    __shared__ typename std::conditional<kFp64, Smem<float, NS, KIJ>, char>::type s32[1];
     const bool warm = kFp64 && !(a.flags & PR_FLAG_NEWTON_FP64_ONLY);
-    if (warm) stage<float, NS, KIJ>(s32[0], a.sp32, a.pair32, a.kij32);
+    if constexpr (kFp64)
+        if (warm) stage<float, NS, KIJ>(s32[0], a.sp32, a.pair32, a.kij32);
     // mixed inversion (FP32 with the FP64 cubic): FP64 tables for the re-solve
     constexpr bool kMixed = sizeof(Real) == 4 && sizeof(RZ) == 8;
     __shared__ typename std::conditional<kMixed, Smem<double, NS, KIJ>, char>::type s64[1];
@@ -609,19 +639,19 @@ __global__ void __launch_bounds__(kBlock) newton_kernel(const NewtonArgs<Real> a
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     if constexpr (kFp64) {
         if (warm) {
-            newton_fp64_queued<NS, KIJ>(a, s, s32[0], stride, a.rtol, 1e-6);
+            newton_fp64_queued<NS, KIJ>(a, s_[0], s32[0], stride, a.rtol, 1e-6);
             return;
         }
         for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += stride) {
             const double hs = __ldg(a.hstar + i), p = __ldg(a.p + i), Tg = __ldg(a.Tg + i);
             Comp<double, NS> c;
-            bool ok = load_comp<double, NS>(c, a.Y, a.ldY, i, a.N, s.sp);
+            bool ok = load_comp<double, NS>(c, a.Y, a.ldY, i, a.N, sp);
             ok = ok && isfinite(hs) && isfinite(Tg) && (p > 0.0) && isfinite(p);
             int st = kBadInput, it = 0;
             double Tres = nan("");
             if (ok) {
                 double cp_last;
-                st = newton_solve<double, double, NS, KIJ>(c, hs, p, fmin(fmax(Tg, kTLo), kTHi), s.sp, s.kij, a.tmid_u,
+                st = newton_solve<double, double, NS, KIJ>(c, hs, p, fmin(fmax(Tg, kTLo), kTHi), sp, kij, a.tmid_u,
                                                            a.max_iter, a.rtol, 1e-6, Tres, it, cp_last);
             }
             a.Tout[i] = Tres;
@@ -663,19 +693,19 @@ __global__ void __launch_bounds__(kBlock) newton_kernel(const NewtonArgs<Real> a
             if (i < a.n) {
                 const float hs = __ldg(a.hstar + i), p = __ldg(a.p + i), Tg = __ldg(a.Tg + i);
                 Comp<float, NS> c;
-                bool ok = load_comp<float, NS>(c, a.Y, a.ldY, i, a.N, s.sp);
+                bool ok = load_comp<float, NS>(c, a.Y, a.ldY, i, a.N, sp);
                 ok = ok && isfinite(hs) && isfinite(Tg) && (p > 0.f) && isfinite(p);
                 int st = kBadInput, it = 0;
                 Temp2 Tres = {__int_as_float(0x7fc00000), 0.f};
                 if (ok) {
                     const float T0 = fminf(fmaxf(Tg, (float)kTLo), (float)kTHi);
                     float cp_last;
-                    st = newton_solve_f32<RZ, NS, KIJ>(c, hs, p, T0, s.sp, s.kij, (float)a.tmid_u, a.max_iter, rtol,
+                    st = newton_solve_f32<RZ, NS, KIJ>(c, hs, p, T0, sp, kij, (float)a.tmid_u, a.max_iter, rtol,
                                                        jump_tol, Tres, it, cp_last);
                     if constexpr (kMixed) {
                         // FP64 where FP32 is least reliable: failed cells, and cells in
                         // the pseudo-boiling band, from the FP32 root (or the guess)
-                        if (st != kOk || cp_last > (float)kPseudoCriticalCp * cp_ideal_mass<float, NS>(c, Tres.h, s.sp)) {
+                        if (st != kOk || cp_last > (float)kPseudoCriticalCp * cp_ideal_mass<float, NS>(c, Tres.h, sp)) {
                             const int e = atomicAdd(&q_n, 1);
                             q_i[e] = i;
                             q_h[e] = st == kOk ? Tres.h : T0;
@@ -720,12 +750,19 @@ void launch_props(const PropsArgs<Real> &a, const void *htab, bool kij, int occ,
     else props_kernel<Real, RZ, NS, false><<<g, kBlock, 0, st>>>(a, make_tab<Real, NS, false>(htab));
 }
 
+template <typename Real, int NS, bool KIJ>
+inline NewtonTab<Real, NS, KIJ> make_newton_tab(const void *htab)
+{
+    if constexpr (NS == 9 && sizeof(Real) == 4) return make_tab<float, 9, KIJ>(htab);
+    else return NoTab{0};
+}
+
 template <typename Real, typename RZ, int NS>
-void launch_newton(const NewtonArgs<Real> &a, bool kij, int occ, int sms, cudaStream_t st)
+void launch_newton(const NewtonArgs<Real> &a, const void *htab, bool kij, int occ, int sms, cudaStream_t st)
 {
     const int g = grid_for(a.n, occ, sms);
-    if (kij) newton_kernel<Real, RZ, NS, true><<<g, kBlock, 0, st>>>(a);
-    else newton_kernel<Real, RZ, NS, false><<<g, kBlock, 0, st>>>(a);
+    if (kij) newton_kernel<Real, RZ, NS, true><<<g, kBlock, 0, st>>>(a, make_newton_tab<Real, NS, true>(htab));
+    else newton_kernel<Real, RZ, NS, false><<<g, kBlock, 0, st>>>(a, make_newton_tab<Real, NS, false>(htab));
 }
 
 // resident CTAs per SM of the property kernels (occ[0..1]: kij off/on) and of
@@ -752,7 +789,7 @@ void occupancy_newton(int occ[2])
     EXT template void launch_props<Real, RZ, NS>(const PropsArgs<Real> &, const void *, bool, int, int, cudaStream_t); \
     EXT template void occupancy_props<Real, RZ, NS>(int *);
 #define PRK_DECLARE_NEWTON(Real, RZ, NS, EXT)                                                             \
-    EXT template void launch_newton<Real, RZ, NS>(const NewtonArgs<Real> &, bool, int, int, cudaStream_t); \
+    EXT template void launch_newton<Real, RZ, NS>(const NewtonArgs<Real> &, const void *, bool, int, int, cudaStream_t); \
     EXT template void occupancy_newton<Real, RZ, NS>(int *);
 #define PRK_DECLARE(Real, RZ, NS, EXT) PRK_DECLARE_PROPS(Real, RZ, NS, EXT) PRK_DECLARE_NEWTON(Real, RZ, NS, EXT)
 
