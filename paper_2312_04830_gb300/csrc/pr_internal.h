@@ -65,6 +65,7 @@ struct pr_ctx {
     // when a constant leaves its range; its resident blocks per SM
     void *h_spfix;
     int occ_spfix;
+    void *h_spshare;     // the FP32 kernel's distinct eps (pr_species.cu SpShare9), 9-species contexts
     // Bilger's mixture fraction: per-species coefficients b_k of the coupling
     // function, then beta_ox and 1 / (beta_fuel - beta_ox) ([n_species + 2])
     double *d_bilger64;

@@ -119,10 +119,12 @@ __device__ __forceinline__ Real corr_factor(const Real *__restrict__ c, int cT, 
 
 // Mixture-averaged D_k [m^2/s] of one valid cell: y its mass fractions
 // (ysum their sum), x its mole fractions (normalised), tab the flat pair table,
-// corr the correction table (cT = 0: none).
-template <typename Real, int NS>
-__device__ __forceinline__ void diffusion_cell(const Real (&y)[NS], const Real (&x)[NS], Real ysum, Real T, Real p,
-                                               int N, const Real *tab, const Real *corr, int cT, int cP, Real (&D)[NS])
+// corr the correction table (cT = 0: none); omega(q, TmB): Omega_D of pair q =
+// k NS + j from T^-B.
+template <typename Real, int NS, typename Omega>
+__device__ __forceinline__ void diffusion_sums(const Real (&y)[NS], const Real (&x)[NS], Real ysum, Real T, Real p,
+                                               int N, const Real *tab, const Real *corr, int cT, int cP, Real (&D)[NS],
+                                               Omega omega)
 {
     const Real *tc = tab, *pc = tab + NS, *ie = tab + 2 * NS, *epsB = ie + NS * NS, *ic = epsB + NS * NS;
     Real Tpc = 0, ppc = 0;
@@ -143,7 +145,7 @@ __device__ __forceinline__ void diffusion_cell(const Real (&y)[NS], const Real (
         for (int j = k + 1; j < NS; ++j) {
             if (j >= N) break;
             const int q = k * NS + j;
-            const Real om = omega_d<Real>(T * ie[q], TmB * epsB[q]);
+            const Real om = omega(q, TmB);
             const Real w = om * ic[q];
             acc[k] = M<Real>::fma(x[j], w, acc[k]);
             acc[j] = M<Real>::fma(x[k], w, acc[j]);
@@ -175,6 +177,15 @@ __device__ __forceinline__ void diffusion_cell(const Real (&y)[NS], const Real (
             D[k] = M<Real>::div(scale, omega_d<Real>(T * ie[q], TmB * epsB[q]) * ic[q]);
         }
     }
+}
+
+template <typename Real, int NS>
+__device__ __forceinline__ void diffusion_cell(const Real (&y)[NS], const Real (&x)[NS], Real ysum, Real T, Real p,
+                                               int N, const Real *tab, const Real *corr, int cT, int cP, Real (&D)[NS])
+{
+    const Real *ie = tab + 2 * NS, *epsB = ie + NS * NS;
+    diffusion_sums<Real, NS>(y, x, ysum, T, p, N, tab, corr, cT, cP, D,
+                             [&](int q, Real TmB) { return omega_d<Real>(T * ie[q], TmB * epsB[q]); });
 }
 
 // h_k^0 / (R T) of one species from its NASA-7 enthalpy record e (molar h =
