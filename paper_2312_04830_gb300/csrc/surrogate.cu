@@ -894,8 +894,9 @@ int num_sms_current()
     return sms[dev] > 0 ? sms[dev] : 148;
 }
 
-// Persistent launch: one CTA per SM (or fewer when there are fewer tiles).
-template <int BN, int EPI>
+// Persistent launch: one CTA per SM, or one CTA pair per two (or fewer when
+// there are fewer tiles).
+template <int BN, int EPI, bool PAIR>
 cudaError_t launch_gemm(const CUtensorMap &ta, const CUtensorMap &tb, GemmArgs a, int m_tiles, int n_tiles,
                         int splits, cudaStream_t st)
 {
@@ -906,44 +907,59 @@ cudaError_t launch_gemm(const CUtensorMap &ta, const CUtensorMap &tb, GemmArgs a
     a.m_tiles = m_tiles;
     a.n_tiles = n_tiles;
     a.splits = splits;
-    const int tiles = m_tiles * n_tiles * splits;
+    const int smem = Cfg<BN, EPI, PAIR>::SMEM;
     if (!dev_ready[dev]) {
         cudaError_t e =
-            cudaFuncSetAttribute(gemm_kernel<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::SMEM);
+            cudaFuncSetAttribute(gemm_kernel<BN, EPI, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         dev_ready[dev] = 1;
     }
-    const int sms = num_sms_current();
-    gemm_kernel<BN, EPI><<<tiles < sms ? tiles : sms, kThreads, Cfg<BN>::SMEM, st>>>(ta, tb, a);
-    return cudaGetLastError();
+    const int units = (PAIR ? (m_tiles + 1) / 2 : m_tiles) * n_tiles * splits;
+    const int most = num_sms_current() / (PAIR ? 2 : 1);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = PAIR ? 2 : 1;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)((PAIR ? 2 : 1) * (units < most ? units : most)), 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = PAIR ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, gemm_kernel<BN, EPI, PAIR>, ta, tb, a);
 }
 
 // Widest N tile (256, 128, 64 or 16) that divides N.
 inline int pick_bn(int N) { return (N % 256 == 0) ? 256 : (N % 128 == 0) ? 128 : (N % 64 == 0) ? 64 : 16; }
 
-// Dispatch on the N tile width.
+// CTA pairs take the N tiles that halve into whole boxes, where there are two
+// M-tiles to pair up and more than one k-block: with one the pair's coupling
+// costs more than its shared loads save (hidden layer, 65536 x 512 x 64: 34 us
+// on pairs, 27 on single CTAs; input gradient 39 and 32).
+template <int BN, int EPI>
+cudaError_t launch_gemm_pair(const CUtensorMap &ta, const CUtensorMap &tb, const GemmArgs &a, int m_tiles, int N,
+                             int splits, cudaStream_t st)
+{
+    return m_tiles >= 2 && a.K > 64 ? launch_gemm<BN, EPI, true>(ta, tb, a, m_tiles, N / BN, splits, st)
+                        : launch_gemm<BN, EPI, false>(ta, tb, a, m_tiles, N / BN, splits, st);
+}
+
+// Dispatch on the N tile width: 256 or 128 (hidden layers' widths are
+// multiples of 128), for the weight gradients also 64 and for the plain GEMM
+// 64 and 16.
 template <int EPI>
 cudaError_t launch_gemm_n(const CUtensorMap &ta, const CUtensorMap &tb, const GemmArgs &a, int m_tiles, int N,
                           int splits, cudaStream_t st)
 {
-    switch (pick_bn(N)) {
-    case 256: return launch_gemm<256, EPI>(ta, tb, a, m_tiles, N / 256, splits, st);
-    case 128: return launch_gemm<128, EPI>(ta, tb, a, m_tiles, N / 128, splits, st);
-    case 64: return launch_gemm<64, EPI>(ta, tb, a, m_tiles, N / 64, splits, st);
-    default: return launch_gemm<16, EPI>(ta, tb, a, m_tiles, N / 16, splits, st);
-    }
-}
-
-// Weight-gradient GEMM with MN-major operands: N tiles of 256, 128 or 64.
-cudaError_t launch_gemm_dw_mn(const CUtensorMap &ta, const CUtensorMap &tb, GemmArgs a, int m_tiles, int N,
-                              int splits, cudaStream_t st)
-{
-    switch (pick_bn(N)) {
-    case 256: return launch_gemm<256, kEpiDwMN>(ta, tb, a, m_tiles, N / 256, splits, st);
-    case 128: return launch_gemm<128, kEpiDwMN>(ta, tb, a, m_tiles, N / 128, splits, st);
-    case 64: return launch_gemm<64, kEpiDwMN>(ta, tb, a, m_tiles, N / 64, splits, st);
-    default: return cudaErrorInvalidValue;
-    }
+    const int bn = pick_bn(N);
+    if (bn == 256) return launch_gemm_pair<256, EPI>(ta, tb, a, m_tiles, N, splits, st);
+    if (bn == 128) return launch_gemm_pair<128, EPI>(ta, tb, a, m_tiles, N, splits, st);
+    if constexpr (EPI == kEpiDw || EPI == kEpiDwMN)
+        if (bn == 64) return launch_gemm<64, EPI, false>(ta, tb, a, m_tiles, N / 64, splits, st);
+    if constexpr (EPI == kEpiDw) return launch_gemm<16, EPI, false>(ta, tb, a, m_tiles, N / 16, splits, st);
+    return cudaErrorInvalidValue;
 }
 
 inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
@@ -1168,8 +1184,8 @@ static pr_status build_maps(sg_model *m)
     const int W = m->width, L = m->hidden;
     const int64_t B = m->max_batch, C = m->chunk;
     bool ok = true;
-    // weights (forward B operands): one box holds a whole N tile of the GEMMs with N = W
-    const uint32_t bw = (uint32_t)pick_bn(W);
+    // weights (forward B operands): boxes of half an N tile of the GEMMs with N = W
+    const uint32_t bw = (uint32_t)b_box_rows(pick_bn(W));
     ok = ok && make_map(&m->tm_w[0], d.wb[0], KIN, W, KIN, bw);
     for (int l = 1; l < L; ++l) ok = ok && make_map(&m->tm_w[l], d.wb[l], W, W, W, bw);
     ok = ok && make_map(&m->tm_w[L], d.wb[L], W, NOP, W, 16);
@@ -1193,12 +1209,12 @@ static pr_status build_maps(sg_model *m)
     ok = ok && make_map(&m->tm_hi[1], d.hi[1], W, C, W, 128);
     // epilogue stores
     for (int l = 0; l < L; ++l) {
-        ok = ok && make_map(&m->ts_h[l], d.h[l], W, B, W, 32);
-        ok = ok && make_map(&m->ts_g[l], d.g[l], W, B, W, 32);
-        ok = ok && make_map(&m->ts_dz[l], d.dz[l], W, B, W, 32);
+        ok = ok && make_map(&m->ts_h[l], d.h[l], W, B, W, 32, 32);
+        ok = ok && make_map(&m->ts_g[l], d.g[l], W, B, W, 32, 32);
+        ok = ok && make_map(&m->ts_dz[l], d.dz[l], W, B, W, 32, 32);
     }
-    ok = ok && make_map(&m->ts_hi[0], d.hi[0], W, C, W, 32);
-    ok = ok && make_map(&m->ts_hi[1], d.hi[1], W, C, W, 32);
+    ok = ok && make_map(&m->ts_hi[0], d.hi[0], W, C, W, 32, 32);
+    ok = ok && make_map(&m->ts_hi[1], d.hi[1], W, C, W, 32, 32);
     // fused inference
     if (m->fused_ok) {
         ok = ok && make_map(&m->tmf_w[0], d.wb[0], KIN, W, KIN, kFusedBN);
@@ -1484,8 +1500,7 @@ static pr_status fwd_bwd(sg_model *m, int64_t B, cudaStream_t st)
         GemmArgs a = base_args(m);
         a.M = (int)B; a.N = W; a.K = (l == 0) ? KIN : W; a.kb_per_split = a.K / 64;
         a.bias = d.master + d.lay[l].b_off;
-        a.out = d.h[l]; a.ldo = W; a.gd = d.g[l]; a.ldg = W;
-        a.tma_out = 1; a.tm_out = m->ts_h[l]; a.tm_gd = m->ts_g[l];
+        a.train = 1; a.last_a = 1; a.flip = l & 1; a.tm_out = m->ts_h[l]; a.tm_gd = m->ts_g[l];
         const CUtensorMap &ta = (l == 0) ? m->tm_x0 : m->tm_h[l - 1];
         e = launch_gemm_n<kEpiHidden>(ta, m->tm_w[l], a, mt, W, 1, st);
         if (e != cudaSuccess) break;
@@ -1499,37 +1514,39 @@ static pr_status fwd_bwd(sg_model *m, int64_t B, cudaStream_t st)
         a.target = d.tgt; a.ldt = d.max_batch;
         a.l1 = m->loss_l1;
         a.loss_scale = (m->loss_l1 ? 1.0f : 2.0f) / (float)(B * d.nout);
-        a.nout = d.nout;
+        a.nout = d.nout; a.flip = L & 1;
         a.out = d.dzo; a.ldo = KIN;
         a.colsum = d.colsum[L]; a.loss_part = d.loss_part;
-        e = launch_gemm<16, kEpiOutLoss>(m->tm_h[L - 1], m->tm_w[L], a, mt, 1, 1, st);
+        e = launch_gemm<16, kEpiOutLoss, false>(m->tm_h[L - 1], m->tm_w[L], a, mt, 1, 1, st);
         if (e != cudaSuccess) { prgb::set_error("loss: %s", cudaGetErrorString(e)); return PR_ECUDA; }
     }
-    // input gradients: dz_{l-1} = (dz_l W_l) * GeLU'(z_{l-1})
-    for (int l = L; l >= 1; --l) {
+    // weight gradients dW_l = dz_l^T h_{l-1} (K = batch, split along K; both
+    // operands read MN-major from the batch-major dz and h) and input
+    // gradients dz_{l-1} = (dz_l W_l) * GeLU'(z_{l-1}), layer by layer: dz_l is
+    // in L2 from the GEMM that wrote it when both read it
+    for (int l = L; l >= 0; --l) {
+        {
+            GemmArgs a = base_args(m);
+            const int mp = d.dw_mpad[l], np = d.lay[l].in_pad;
+            a.M = mp; a.Mpad = mp; a.N = np; a.K = (int)B; a.kb_per_split = d.dw_kps[l];
+            a.partial = d.partial[l];
+            a.last_a = (l == 0); a.last_b = 1;
+            const int splits = ceil_div(ceil_div(B, 64), d.dw_kps[l]);
+            const CUtensorMap &ta = (l == L) ? m->tmn_dzo : m->tmn_dz[l];
+            const CUtensorMap &tb = (l == 0) ? m->tmn_x0 : m->tmn_h[l - 1];
+            e = launch_gemm_n<kEpiDwMN>(ta, tb, a, mp / 128, np, splits, st);
+            if (e != cudaSuccess) { prgb::set_error("dw: %s", cudaGetErrorString(e)); return PR_ECUDA; }
+            m->last_splits[l] = splits;
+        }
+        if (l == 0) break;
         GemmArgs a = base_args(m);
         a.M = (int)B; a.N = W; a.K = (l == L) ? KIN : W; a.kb_per_split = a.K / 64;
-        a.gd = d.g[l - 1]; a.ldg = W;
-        a.out = d.dz[l - 1]; a.ldo = W;
-        a.tma_out = 1; a.tm_out = m->ts_dz[l - 1];
+        a.tm_out = m->ts_dz[l - 1]; a.tm_gd = m->ts_g[l - 1];
         a.colsum = d.colsum[l - 1];
+        a.last_a = 1; a.flip = l & 1;
         const CUtensorMap &ta = (l == L) ? m->tm_dzo : m->tm_dz[l];
         e = launch_gemm_n<kEpiDx>(ta, m->tm_wt[l], a, mt, W, 1, st);
         if (e != cudaSuccess) { prgb::set_error("dx: %s", cudaGetErrorString(e)); return PR_ECUDA; }
-    }
-    // weight gradients: dW_l = dz_l^T h_{l-1}, K = batch, split along K; both
-    // operands read MN-major from the batch-major dz and h
-    for (int l = 0; l <= L; ++l) {
-        GemmArgs a = base_args(m);
-        const int mp = d.dw_mpad[l], np = d.lay[l].in_pad;
-        a.M = mp; a.Mpad = mp; a.N = np; a.K = (int)B; a.kb_per_split = d.dw_kps[l];
-        a.partial = d.partial[l];
-        const int splits = ceil_div(ceil_div(B, 64), d.dw_kps[l]);
-        const CUtensorMap &ta = (l == L) ? m->tmn_dzo : m->tmn_dz[l];
-        const CUtensorMap &tb = (l == 0) ? m->tmn_x0 : m->tmn_h[l - 1];
-        e = launch_gemm_dw_mn(ta, tb, a, mp / 128, np, splits, st);
-        if (e != cudaSuccess) { prgb::set_error("dw: %s", cudaGetErrorString(e)); return PR_ECUDA; }
-        m->last_splits[l] = splits;
     }
     return PR_OK;
 }
@@ -1691,8 +1708,7 @@ pr_status surrogate_infer(sg_model *m, int64_t n, const float *T, const float *p
             GemmArgs a = base_args(m);
             a.M = (int)mc; a.N = W; a.K = (l == 0) ? KIN : W; a.kb_per_split = a.K / 64;
             a.bias = d.master + d.lay[l].b_off;
-            a.out = d.hi[l & 1]; a.ldo = W;
-            a.tma_out = 1; a.tm_out = m->ts_hi[l & 1];
+            a.tm_out = m->ts_hi[l & 1];
             const CUtensorMap &ta = (l == 0) ? m->tm_xi : m->tm_hi[(l - 1) & 1];
             PR_CUDA_TRY((launch_gemm_n<kEpiHidden>(ta, m->tm_w[l], a, mt, W, 1, st)));
         }
@@ -1705,7 +1721,7 @@ pr_status surrogate_infer(sg_model *m, int64_t n, const float *T, const float *p
             a.add_h = (d.mode != SG_MODE_FORWARD) ? nullptr : d.hig;
             a.log_mask = log_mask_of(d.mode, d.outputs);
             a.nout = d.nout;
-            PR_CUDA_TRY((launch_gemm<16, kEpiOutPhys>(m->tm_hi[(L - 1) & 1], m->tm_w[L], a, mt, 1, 1, st)));
+            PR_CUDA_TRY((launch_gemm<16, kEpiOutPhys, false>(m->tm_hi[(L - 1) & 1], m->tm_w[L], a, mt, 1, 1, st)));
         }
         if (m->time_mlp) PR_CUDA_TRY(cudaEventRecord(tm1, st));
         const float ctol = (d.mode == SG_MODE_FORWARD) ? m->conf_tol : 0.f;
@@ -1979,7 +1995,7 @@ pr_status mlp_gemm_bf16(int64_t M, int64_t N, int64_t K, const void *A, int64_t 
     PR_CHECK_ARG(prgb::aligned(A, 16) && prgb::aligned(B, 16) && prgb::aligned(D, 16), "mlp_gemm_bf16: 16-byte alignment");
     const int bn = pick_bn((int)N);
     CUtensorMap ta, tb;
-    if (!make_map(&ta, A, K, M, lda, 128) || !make_map(&tb, B, K, N, ldb, bn)) {
+    if (!make_map(&ta, A, K, M, lda, 128) || !make_map(&tb, B, K, N, ldb, b_box_rows(bn))) {
         prgb::set_error("mlp_gemm_bf16: tensor map encoding failed");
         return PR_ECUDA;
     }
@@ -1989,11 +2005,7 @@ pr_status mlp_gemm_bf16(int64_t M, int64_t N, int64_t K, const void *A, int64_t 
     a.partial = D;
     a.err = err_flag;
     cudaStream_t st = (cudaStream_t)stream;
-    const int gx = ceil_div(M, 128), gy = (int)(N / bn);
-    cudaError_t e;
-    e = launch_gemm_n<kEpiDw>(ta, tb, a, gx, (int)N, 1, st);
-    (void)gy;
-    PR_CUDA_TRY(e);
+    PR_CUDA_TRY((launch_gemm_n<kEpiDw>(ta, tb, a, ceil_div(M, 128), (int)N, 1, st)));
     return PR_OK;
 }
 
