@@ -470,6 +470,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
     umma::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     bool fail = false;
+    umma::pdl_wait();      // (no global memory is touched above)
+    umma::pdl_release();
 
     if (warp == 0) {
         // ------------------------------------------- TMA producer (each CTA)

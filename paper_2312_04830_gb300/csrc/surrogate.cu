@@ -249,6 +249,8 @@ __device__ __forceinline__ void write_bf16_copies(const SgDev &d, const ParamRef
 // max out_pad / 32, L), block 32 x 8.
 __global__ void transpose_w_kernel(SgDev d)
 {
+    umma::pdl_wait();
+    umma::pdl_release();
     __shared__ __nv_bfloat16 tile[32][33];
     const int l = blockIdx.z + 1;
     const LayerLayout &Ly = d.lay[l];
@@ -267,9 +269,36 @@ __global__ void transpose_w_kernel(SgDev d)
     }
 }
 
+// Launch of a training step's kernel: its blocks may take their places (and,
+// in a GEMM, set up barriers and tensor memory) while the kernel before it
+// drains; each waits (pdl_wait) before it touches global memory.  A step is 20
+// launches with 8 to 10 us each to launch, fill and drain: 512 x 4, batch
+// 65536, 600 us a step launched one after the other, 557 so.  `cluster` CTAs
+// to a cluster.
+template <class... P, class... A>
+cudaError_t launch_step(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, int cluster, cudaStream_t st,
+                        const A &...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 void launch_transpose_w(const SgDev &d, cudaStream_t st)
 {
-    transpose_w_kernel<<<dim3(d.width / 32, d.width / 32, d.hidden), dim3(32, 8), 0, st>>>(d);
+    launch_step(transpose_w_kernel, dim3(d.width / 32, d.width / 32, d.hidden), dim3(32, 8), 0, 1, st, d);
 }
 
 __global__ void refresh_bf16_kernel(SgDev d)
@@ -392,6 +421,8 @@ __device__ __forceinline__ void split_hi_lo(const float (&v)[16], float (&lo)[16
 __global__ void prep_train_kernel(SgDev d, int64_t B, int64_t n_pool, const float *x, int64_t ldx, const float *y,
                                   int64_t ldy, uint64_t sample_seed)
 {
+    umma::pdl_wait();
+    umma::pdl_release();
     const float *nm = d.norm;
     for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < B; r += (int64_t)gridDim.x * blockDim.x) {
         int64_t src = r;
@@ -674,6 +705,8 @@ __global__ void __launch_bounds__(128) fallback_species_kernel(const int32_t *li
 // of dz (nct of them), lanes striding over the tiles.
 __global__ void bias_grad_kernel(SgDev d, int64_t nct)
 {
+    umma::pdl_wait();
+    umma::pdl_release();
     const int lane = threadIdx.x & 31;
     const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int l = (int)(wid / d.width), o = (int)(wid % d.width);
@@ -754,6 +787,8 @@ __device__ __forceinline__ void partial_sum4(const float *pp, int64_t plane, int
 __global__ void __launch_bounds__(256) adam_kernel(SgDev d, float lr, float b1, float b2, float eps, int t,
                                                    int export_only, float *grad_out)
 {
+    umma::pdl_wait();
+    umma::pdl_release();
     const int64_t e = 4 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
     if (e >= d.n_master) return;
     const float bc1 = 1.f - powf(b1, (float)t), bc2 = 1.f - powf(b2, (float)t);
@@ -812,6 +847,8 @@ inline int adam_blocks(const SgDev &d) { return (int)((d.n_master + 1023) / 1024
 
 __global__ void loss_final_kernel(const float *part, int64_t nct, float scale, float *loss_out)
 {
+    umma::pdl_wait();
+    umma::pdl_release();
     __shared__ float sh[256];
     float s = 0.f;
     for (int64_t c = threadIdx.x; c < nct; c += blockDim.x) s += part[c];
@@ -916,19 +953,8 @@ cudaError_t launch_gemm(const CUtensorMap &ta, const CUtensorMap &tb, GemmArgs a
     }
     const int units = (PAIR ? (m_tiles + 1) / 2 : m_tiles) * n_tiles * splits;
     const int most = num_sms_current() / (PAIR ? 2 : 1);
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = PAIR ? 2 : 1;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)((PAIR ? 2 : 1) * (units < most ? units : most)), 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = PAIR ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, gemm_kernel<BN, EPI, PAIR>, ta, tb, a);
+    return launch_step(gemm_kernel<BN, EPI, PAIR>, dim3((unsigned)((PAIR ? 2 : 1) * (units < most ? units : most))),
+                       dim3(kThreads), smem, PAIR ? 2 : 1, st, ta, tb, a);
 }
 
 // Widest N tile (256, 128, 64 or 16) that divides N.
@@ -1562,24 +1588,22 @@ static pr_status train_common(sg_model *m, int64_t batch, int64_t n_pool, const 
     cudaStream_t st = (cudaStream_t)stream;
     SgDev &d = m->dev;
     const int blocks = ceil_div(batch, 256);
-    prep_train_kernel<<<blocks < 2048 ? blocks : 2048, 256, 0, st>>>(d, batch, n_pool, x, ldx, y, ldy, seed);
-    PR_CUDA_TRY(cudaGetLastError());
+    PR_CUDA_TRY(launch_step(prep_train_kernel, dim3(blocks < 2048 ? blocks : 2048), dim3(256), 0, 1, st, d, batch, n_pool,
+                            x, ldx, y, ldy, seed));
     // the dw GEMMs split K over dw_kps k-blocks: make sure the splits fit the batch
     for (int l = 0; l <= m->hidden; ++l) d.dw_splits[l] = ceil_div(ceil_div(batch, 64), d.dw_kps[l]);
     pr_status s = fwd_bwd(m, batch, st);
     if (s) return s;
     const int64_t nct = batch / 128;
-    if (grad_out) {
-        bias_grad_kernel<<<(int)(((int64_t)(m->hidden + 1) * m->width * 32 + 255) / 256), 256, 0, st>>>(d, nct);
-        adam_kernel<<<adam_blocks(d), 256, 0, st>>>(d, 0.f, 0.9f, 0.999f, 1e-8f, 1, 1, grad_out);
-    } else {
-        m->step += 1;
-        bias_grad_kernel<<<(int)(((int64_t)(m->hidden + 1) * m->width * 32 + 255) / 256), 256, 0, st>>>(d, nct);
-        adam_kernel<<<adam_blocks(d), 256, 0, st>>>(d, lr, 0.9f, 0.999f, 1e-8f, (int)m->step, 0, nullptr);
-        launch_transpose_w(d, st);
-    }
+    PR_CUDA_TRY(launch_step(bias_grad_kernel, dim3((unsigned)(((int64_t)(m->hidden + 1) * m->width * 32 + 255) / 256)),
+                            dim3(256), 0, 1, st, d, nct));
+    if (!grad_out) m->step += 1;
+    PR_CUDA_TRY(launch_step(adam_kernel, dim3(adam_blocks(d)), dim3(256), 0, 1, st, d, grad_out ? 0.f : lr, 0.9f, 0.999f,
+                            1e-8f, grad_out ? 1 : (int)m->step, grad_out ? 1 : 0, grad_out));
+    if (!grad_out) launch_transpose_w(d, st);
     float *lo = loss_out ? loss_out : m->d_loss;
-    loss_final_kernel<<<1, 256, 0, st>>>(d.loss_part, nct, 1.0f / (float)(batch * d.nout), lo);
+    PR_CUDA_TRY(launch_step(loss_final_kernel, dim3(1), dim3(256), 0, 1, st, d.loss_part, nct,
+                            1.0f / (float)(batch * d.nout), lo));
     PR_CUDA_TRY(cudaGetLastError());
     return PR_OK;
 }

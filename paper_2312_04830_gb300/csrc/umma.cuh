@@ -18,6 +18,15 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p)
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// ------------------------------------------- programmatic dependent launch
+// A kernel launched with programmatic stream serialisation may start once
+// every block of its predecessor has called pdl_release (or has ended); past
+// pdl_wait the predecessor has ended and what it wrote is visible.  Every
+// thread of such a kernel that touches global memory waits first, so a kernel
+// that has ended had all its predecessors end before it.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ------------------------------------------------------------ mbarriers
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
 {

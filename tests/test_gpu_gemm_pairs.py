@@ -65,3 +65,33 @@ def test_pairs_in_training_and_layerwise_inference(ctx, cuda, width):
             assert np.array_equal(out[:, s].cpu().numpy(), one.cpu().numpy(), equal_nan=True), (n, r)
     sg.sync_status()
     sg.close()
+
+
+def test_captured_steps(ctx, cuda):
+    """Training steps under stream capture: two steps in a graph (learning rate
+    zero, so every step has the same loss) give the loss of one outside it."""
+    import torch
+    from paper_2312_04830_gb300 import binding
+    g = torch.Generator(device="cpu").manual_seed(9)
+    x = torch.rand(11, 1024, generator=g) + 0.1
+    x[0], x[1] = 300.0 + 2000.0 * x[0], 1e7 * x[1]
+    x[2:] /= x[2:].sum(0)
+    x, y = x.to(cuda), torch.randn(6, 1024, generator=g).to(cuda)
+    sg = binding.Surrogate(ctx, width=256, hidden_layers=2, max_batch=1024, infer_chunk=1024, seed=3)
+    sg.fit_normalization(x, y)
+    loss = torch.zeros(2, device=cuda)
+    torch.cuda.synchronize()
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        sg.train_step(x, y, 1024, 0.0, sample_seed=5, loss_out=loss, stream=st)
+        st.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=st):
+            for _ in range(2):
+                sg.train_step(x, y, 1024, 0.0, sample_seed=5, loss_out=loss[1:], stream=st)
+        for _ in range(3):
+            graph.replay()
+    torch.cuda.synchronize()
+    assert float(loss[0]) == float(loss[1]) > 0.0
+    sg.sync_status()
+    sg.close()
