@@ -207,7 +207,8 @@ void launch_newton_fix(const NewtonArgs<double> &a, const Fix9 &t, const void *h
         newton_warm_kernel<<<grid_for(a.n, occ[0], sms), kBlock, 0, st>>>(a, make_tab<float, 9, false>(htab32));
         newton_fix_kernel<true><<<grid_for(a.n, occ[1], sms), kBlock, 0, st>>>(a, t);
     } else {
-        newton_fix_kernel<false><<<grid_for(a.n, occ[2], sms), kBlock, 0, st>>>(a, t);
+        const int b = block_for(a.n, sms);
+        newton_fix_kernel<false><<<grid_for(a.n, occ[2], sms, b), b, 0, st>>>(a, t);
     }
 }
 

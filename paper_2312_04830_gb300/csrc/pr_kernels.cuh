@@ -734,9 +734,16 @@ __global__ void __launch_bounds__(kBlock) newton_kernel(const __grid_constant__ 
 
 
 // ------------------------------------------------------------- launchers
-inline int grid_for(int64_t n, int occ, int sms)
+// Threads per block: one warp while that gives every block an SM of its own,
+// then two.  A small call is as long as its busiest SM, whose FP64 pipe takes
+// 16 cycles per warp instruction: 1000 cells of FP64 properties 43.7 -> 41.7 us
+// a call, most of it one cell's dependent chain (38 us in the kernel with one
+// warp an SM, 41 with two, 44 with four).
+inline int block_for(int64_t n, int sms) { return n <= 32 * (int64_t)sms ? 32 : n <= 64 * (int64_t)sms ? 64 : kBlock; }
+
+inline int grid_for(int64_t n, int occ, int sms, int block = kBlock)
 {
-    int64_t need = (n + kBlock - 1) / kBlock;
+    int64_t need = (n + block - 1) / block;
     int64_t cap = (int64_t)occ * sms;
     return (int)(need < cap ? need : cap);
 }
@@ -745,9 +752,9 @@ inline int grid_for(int64_t n, int occ, int sms)
 template <typename Real, typename RZ, int NS>
 void launch_props(const PropsArgs<Real> &a, const void *htab, bool kij, int occ, int sms, cudaStream_t st)
 {
-    const int g = grid_for(a.n, occ, sms);
-    if (kij) props_kernel<Real, RZ, NS, true><<<g, kBlock, 0, st>>>(a, make_tab<Real, NS, true>(htab));
-    else props_kernel<Real, RZ, NS, false><<<g, kBlock, 0, st>>>(a, make_tab<Real, NS, false>(htab));
+    const int b = block_for(a.n, sms), g = grid_for(a.n, occ, sms, b);
+    if (kij) props_kernel<Real, RZ, NS, true><<<g, b, 0, st>>>(a, make_tab<Real, NS, true>(htab));
+    else props_kernel<Real, RZ, NS, false><<<g, b, 0, st>>>(a, make_tab<Real, NS, false>(htab));
 }
 
 template <typename Real, int NS, bool KIJ>
@@ -760,9 +767,9 @@ inline NewtonTab<Real, NS, KIJ> make_newton_tab(const void *htab)
 template <typename Real, typename RZ, int NS>
 void launch_newton(const NewtonArgs<Real> &a, const void *htab, bool kij, int occ, int sms, cudaStream_t st)
 {
-    const int g = grid_for(a.n, occ, sms);
-    if (kij) newton_kernel<Real, RZ, NS, true><<<g, kBlock, 0, st>>>(a, make_newton_tab<Real, NS, true>(htab));
-    else newton_kernel<Real, RZ, NS, false><<<g, kBlock, 0, st>>>(a, make_newton_tab<Real, NS, false>(htab));
+    const int b = block_for(a.n, sms), g = grid_for(a.n, occ, sms, b);
+    if (kij) newton_kernel<Real, RZ, NS, true><<<g, b, 0, st>>>(a, make_newton_tab<Real, NS, true>(htab));
+    else newton_kernel<Real, RZ, NS, false><<<g, b, 0, st>>>(a, make_newton_tab<Real, NS, false>(htab));
 }
 
 // resident CTAs per SM of the property kernels (occ[0..1]: kij off/on) and of
