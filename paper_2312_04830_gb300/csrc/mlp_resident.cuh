@@ -212,19 +212,23 @@ __global__ void __launch_bounds__(kResThreads, 1) mlp_resident_kernel(const __gr
         umma::fence_mbar_init();
         umma::tma_prefetch_desc(&a.tm_x);
     }
-    for (int e = threadIdx.x; e < L * W + kResOutBN; e += blockDim.x) {
-        const int l = (e < L * W) ? e / W : L;
-        const int n = (e < L * W) ? e - l * W : e - L * W;
-        sbias[e] = __ldg(a.bias[l] + n);
-    }
     __syncthreads();
     if (warp == 1) {
         umma::tmem_alloc_pair(tmem_slot, 512);
         umma::tmem_relinquish_pair();
     }
+    for (int e = threadIdx.x; e < L * W + kResOutBN; e += blockDim.x) {
+        const int l = (e < L * W) ? e / W : L;
+        const int n = (e < L * W) ? e - l * W : e - L * W;
+        sbias[e] = __ldg(a.bias[l] + n);
+    }
     umma::tc_fence_before();
     __syncthreads();
     umma::cluster_sync();   // both CTAs' barriers initialised before any copy or MMA signals them
+    // the kernel before this one writes the inputs (the biases above are older
+    // than its start: it is launched in stream order)
+    umma::pdl_wait();
+    umma::pdl_release();
     umma::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     bool fail = false;

@@ -269,12 +269,13 @@ __global__ void transpose_w_kernel(SgDev d)
     }
 }
 
-// Launch of a training step's kernel: its blocks may take their places (and,
+// Launch of a kernel of a training step or an inference call: its blocks may take their places (and,
 // in a GEMM, set up barriers and tensor memory) while the kernel before it
 // drains; each waits (pdl_wait) before it touches global memory.  A step is 20
 // launches with 8 to 10 us each to launch, fill and drain: 512 x 4, batch
-// 65536, 600 us a step launched one after the other, 557 so.  `cluster` CTAs
-// to a cluster.
+// 65536, 600 us a step launched one after the other, 557 so; an inference call
+// of 20011 cells (256 x 3, in a graph) 37.8 us and 34.8.  `cluster` CTAs to a
+// cluster.
 template <class... P, class... A>
 cudaError_t launch_step(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, int cluster, cudaStream_t st,
                         const A &...args)
@@ -447,6 +448,7 @@ __global__ void prep_train_kernel(SgDev d, int64_t B, int64_t n_pool, const floa
 __global__ void prep_infer_kernel(SgDev d, int64_t r0, int64_t mc, const float *T, const float *p, const float *Y,
                                   int64_t ldY, uint8_t *flags, uint8_t *cflags, int32_t *list, unsigned int *count)
 {
+    umma::pdl_release();   // (launched in stream order, so nothing to wait for)
     const float *nm = d.norm;
     const float *lo = nm + 2 * NIN + 2 * NOUT6, *hi = lo + NIN;
     for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < mc; r += (int64_t)gridDim.x * blockDim.x) {
@@ -509,6 +511,8 @@ __global__ void __launch_bounds__(256) confidence_kernel(SgDev d, int64_t r0, in
         for (int j = threadIdx.x; j < (int)(9 * sizeof(SpeciesRec<float>) / 4); j += blockDim.x) dst[j] = src[j];
         for (int j = threadIdx.x; j < 81; j += blockDim.x) s_pair[j] = d.pair32[j];
     }
+    umma::pdl_wait();   // (the tables are older than the call)
+    umma::pdl_release();
     __syncthreads();
     const bool fwd = d.mode == SG_MODE_FORWARD;
     for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < mc; r += (int64_t)gridDim.x * blockDim.x) {
@@ -572,6 +576,7 @@ __global__ void __launch_bounds__(128) fallback_kernel(const int32_t *list, cons
         for (int j = threadIdx.x; j < (int)(NS * sizeof(SpeciesRec<double>) / 8); j += blockDim.x) dst[j] = src[j];
         for (int j = threadIdx.x; j < NS * NS; j += blockDim.x) { s_pair[j] = pair[j]; s_kij[j] = kij[j]; }
     }
+    umma::pdl_wait();   // (the tables are older than the call)
     __syncthreads();
     const unsigned int n = *count;
     for (unsigned int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x)
@@ -600,6 +605,7 @@ __global__ void __launch_bounds__(128) fallback_inverse_kernel(const int32_t *li
         for (int j = threadIdx.x; j < (int)(NS * sizeof(SpeciesRec<double>) / 8); j += blockDim.x) dst[j] = src[j];
         for (int j = threadIdx.x; j < NS * NS; j += blockDim.x) { s_pair[j] = pair[j]; s_kij[j] = kij[j]; }
     }
+    umma::pdl_wait();   // (the tables are older than the call)
     __syncthreads();
     const unsigned int n = *count;
     for (unsigned int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
@@ -664,6 +670,7 @@ __global__ void __launch_bounds__(128) fallback_species_kernel(const int32_t *li
         for (int j = threadIdx.x; j < NS * NS; j += blockDim.x) s_kij[j] = kij[j];
         for (int j = threadIdx.x; j < 2 * NS + 3 * NS * NS; j += blockDim.x) s_tab[j] = dtab[j];
     }
+    umma::pdl_wait();   // (the tables are older than the call)
     __syncthreads();
     const unsigned int n = *count;
     for (unsigned int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
@@ -1176,21 +1183,12 @@ cudaError_t launch_resident(const ResidentArgs &ra, int pairs, cudaStream_t st)
 {
     const int R = (ra.M + 255) / 256;
     const int g = R < pairs ? R : pairs;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)(2 * g), 1, 1);
-    cfg.blockDim = dim3(kResThreads, 1, 1);
-    cfg.dynamicSmemBytes = ResCfg::smem_bytes(ra.L, ra.W, ResCfg::stages(ra.L, ra.W));
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (ResCfg::stages(ra.L, ra.W) == 3) return cudaLaunchKernelEx(&cfg, mlp_resident_kernel<512, 3>, ra);
-    return ra.W == 256 ? cudaLaunchKernelEx(&cfg, mlp_resident_kernel<256, 4>, ra)
-                       : cudaLaunchKernelEx(&cfg, mlp_resident_kernel<512, 4>, ra);
+    const int stages = ResCfg::stages(ra.L, ra.W);
+    void (*kernel)(const ResidentArgs) = stages == 3   ? mlp_resident_kernel<512, 3>
+                                         : ra.W == 256 ? mlp_resident_kernel<256, 4>
+                                                       : mlp_resident_kernel<512, 4>;
+    return launch_step(kernel, dim3((unsigned)(2 * g)), dim3(kResThreads), ResCfg::smem_bytes(ra.L, ra.W, stages), 2, st,
+                       ra);
 }
 
 GemmArgs base_args(sg_model *m)
@@ -1751,43 +1749,29 @@ pr_status surrogate_infer(sg_model *m, int64_t n, const float *T, const float *p
         const float ctol = (d.mode == SG_MODE_FORWARD) ? m->conf_tol : 0.f;
         const float ttol = (d.outputs == SG_OUT_PROPS) ? m->tr_tol : 0.f;
         if (ctol > 0.f || ttol > 0.f) {
-            confidence_kernel<<<pb < 4096 ? pb : 4096, 256, 0, st>>>(d, r0, mc, T, p, Y, ldY, out, ldo, ctol, ttol,
-                                                                     used_fallback, m->d_flags, m->d_list, m->d_count);
-            PR_CUDA_TRY(cudaGetLastError());
+            PR_CUDA_TRY(launch_step(confidence_kernel, dim3(pb < 4096 ? pb : 4096), dim3(256), 0, 1, st, d, r0, mc, T, p, Y,
+                                    ldY, out, ldo, ctol, ttol, used_fallback, m->d_flags, m->d_list, m->d_count));
         }
         // FP64 Peng-Robinson for the cells outside the training hull (and the low-confidence ones)
         const int fb = ctx->num_sms * 4;
         const SpeciesRec<double> *sp64 = (const SpeciesRec<double> *)ctx->d_sp64;
         const int sel = (d.outputs >= SG_OUT_SINGLE) ? d.outputs - SG_OUT_SINGLE : -1;
-        if (d.outputs == SG_OUT_DK || d.outputs == SG_OUT_HK) {
-            if (ctx->has_kij)
-                fallback_species_kernel<9, true><<<fb, 128, 0, st>>>(m->d_list, m->d_count, r0, T, p, Y, ldY, out,
-                                                                     ldo, sp64, ctx->d_kij64, ctx->d_dtab64,
-                                                                     ctx->d_corr64, ctx->corr_nT, ctx->corr_nP,
-                                                                     ctx->n_species, d.outputs);
-            else
-                fallback_species_kernel<9, false><<<fb, 128, 0, st>>>(m->d_list, m->d_count, r0, T, p, Y, ldY, out,
-                                                                      ldo, sp64, ctx->d_kij64, ctx->d_dtab64,
-                                                                      ctx->d_corr64, ctx->corr_nT, ctx->corr_nP,
-                                                                      ctx->n_species, d.outputs);
-        } else if (d.mode != SG_MODE_FORWARD) {
-            if (ctx->has_kij)
-                fallback_inverse_kernel<9, true><<<fb, 128, 0, st>>>(m->d_list, m->d_count, r0, T, p, Y, ldY, out,
-                                                                     ldo, sp64, ctx->d_pair64, ctx->d_kij64,
-                                                                     ctx->n_species, ctx->flags, sel);
-            else
-                fallback_inverse_kernel<9, false><<<fb, 128, 0, st>>>(m->d_list, m->d_count, r0, T, p, Y, ldY, out,
-                                                                      ldo, sp64, ctx->d_pair64, ctx->d_kij64,
-                                                                      ctx->n_species, ctx->flags, sel);
-        } else if (ctx->has_kij)
-            fallback_kernel<9, true><<<fb, 128, 0, st>>>(m->d_list, m->d_count, r0, T, p, Y, ldY, out, ldo,
-                                                         (const SpeciesRec<double> *)ctx->d_sp64, ctx->d_pair64,
-                                                         ctx->d_kij64, ctx->n_species, ctx->flags, ctx->tmid_u);
+        auto fall_back = [&](auto kernel, auto... args) {
+            return launch_step(kernel, dim3(fb), dim3(128), 0, 1, st, m->d_list, m->d_count, r0, T, p, Y, ldY, out, ldo,
+                               sp64, args...);
+        };
+        const bool kij = ctx->has_kij;
+        cudaError_t fe;
+        if (d.outputs == SG_OUT_DK || d.outputs == SG_OUT_HK)
+            fe = fall_back(kij ? fallback_species_kernel<9, true> : fallback_species_kernel<9, false>, ctx->d_kij64,
+                           ctx->d_dtab64, ctx->d_corr64, ctx->corr_nT, ctx->corr_nP, ctx->n_species, d.outputs);
+        else if (d.mode != SG_MODE_FORWARD)
+            fe = fall_back(kij ? fallback_inverse_kernel<9, true> : fallback_inverse_kernel<9, false>, ctx->d_pair64,
+                           ctx->d_kij64, ctx->n_species, ctx->flags, sel);
         else
-            fallback_kernel<9, false><<<fb, 128, 0, st>>>(m->d_list, m->d_count, r0, T, p, Y, ldY, out, ldo,
-                                                          (const SpeciesRec<double> *)ctx->d_sp64, ctx->d_pair64,
-                                                          ctx->d_kij64, ctx->n_species, ctx->flags, ctx->tmid_u);
-        PR_CUDA_TRY(cudaGetLastError());
+            fe = fall_back(kij ? fallback_kernel<9, true> : fallback_kernel<9, false>, ctx->d_pair64, ctx->d_kij64,
+                           ctx->n_species, ctx->flags, ctx->tmid_u);
+        PR_CUDA_TRY(fe);
     }
     return PR_OK;
 }
