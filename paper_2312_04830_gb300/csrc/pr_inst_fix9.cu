@@ -136,6 +136,7 @@ __global__ void __launch_bounds__(kBlock, 4) newton_fix_kernel(const __grid_cons
     __shared__ unsigned char q_first[2 * kBlock];
     if (threadIdx.x == 0) q_n = 0;
     stage<float, 9, false>(s32, a.sp32, a.pair32, a.kij32);   // ends with a barrier
+    auto finish = [&](int e) { newton_finish9(a, q_i[e], q_T[e], q_first[e] != 0, q_h[e], q_cp[e]); };
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.n; base += stride) {
         const int64_t i = base + threadIdx.x;
@@ -167,19 +168,9 @@ __global__ void __launch_bounds__(kBlock, 4) newton_fix_kernel(const __grid_cons
                 newton_fix_cell(a, t, i, T, wok ? cp32 : 0.f, s32.sp, &q_n, q_i, q_T, q_h, q_cp, q_first, isfinite(Tg));
             }
         }
-        __syncthreads();
-        while (q_n >= (int)blockDim.x) {
-            const int e = q_n - (int)blockDim.x + (int)threadIdx.x;
-            newton_finish9(a, q_i[e], q_T[e], q_first[e] != 0, q_h[e], q_cp[e]);
-            __syncthreads();
-            if (threadIdx.x == 0) q_n -= (int)blockDim.x;
-            __syncthreads();
-        }
+        queue_round(&q_n, (int)threadIdx.x, (int)blockDim.x, finish);
     }
-    if ((int)threadIdx.x < q_n) {
-        const int e = threadIdx.x;
-        newton_finish9(a, q_i[e], q_T[e], q_first[e] != 0, q_h[e], q_cp[e]);
-    }
+    queue_rest(&q_n, (int)threadIdx.x, finish);
 }
 
 // [a, a + na) and [b, b + nb) share a byte

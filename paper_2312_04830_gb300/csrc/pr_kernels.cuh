@@ -15,6 +15,7 @@
 #include <type_traits>
 
 #include "pr_device.cuh"
+#include "pr_queue.cuh"
 
 namespace prk {
 
@@ -594,15 +595,9 @@ __device__ __forceinline__ void newton_fp64_queued(const NewtonArgs<double> &a, 
                 }
             }
         }
-        __syncthreads();
-        while (q_n >= (int)blockDim.x) {
-            finish(q_n - (int)blockDim.x + (int)threadIdx.x);
-            __syncthreads();
-            if (threadIdx.x == 0) q_n -= (int)blockDim.x;
-            __syncthreads();
-        }
+        queue_round(&q_n, (int)threadIdx.x, (int)blockDim.x, finish);
     }
-    if ((int)threadIdx.x < q_n) finish((int)threadIdx.x);
+    queue_rest(&q_n, (int)threadIdx.x, finish);
 }
 
 // The FP32 and mixed kernels of up to 9 species take their FP32 tables in the
@@ -718,17 +713,9 @@ __global__ void __launch_bounds__(kBlock) newton_kernel(const __grid_constant__ 
                 a.status[i] = st;
                 if (a.iters) a.iters[i] = it;
             }
-            if constexpr (kMixed) {
-                __syncthreads();
-                while (q_n >= (int)blockDim.x) {
-                    finish(q_n - (int)blockDim.x + (int)threadIdx.x);
-                    __syncthreads();
-                    if (threadIdx.x == 0) q_n -= (int)blockDim.x;
-                    __syncthreads();
-                }
-            }
+            if constexpr (kMixed) queue_round(&q_n, (int)threadIdx.x, (int)blockDim.x, finish);
         }
-        if (kMixed && (int)threadIdx.x < q_n) finish((int)threadIdx.x);
+        if constexpr (kMixed) queue_rest(&q_n, (int)threadIdx.x, finish);
     }
 }
 
