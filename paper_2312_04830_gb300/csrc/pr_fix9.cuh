@@ -110,9 +110,13 @@ __device__ __forceinline__ int fix9_comp(const Fix9 &t, const double (&y)[9], Fi
     const int z = __clzll((long long)s);
     const uint64_t sn = s << z;                     // s > 0: the mass fractions sum to 1
     const uint64_t r = i64::rcp_m(sn);              // 2^64 / (sn / 2^63)
+    // r is at most two units high (its residual is rounded up by less than one
+    // unit of 2^-63): with two taken off, x of a species alone in its cell
+    // stays below 2^63, the end of xh
+    const uint64_t rx = r - 2;
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-        const uint64_t x = i64::mulhi(n[k] << z, r);   // units 2^-63, at most 2^63
+        const uint64_t x = i64::mulhi(n[k] << z, rx);   // units 2^-63
         c.xh[k] = (int32_t)(x >> 32);
         c.xl[k] = (int32_t)(i64::lo32(x) >> 1);
     }
