@@ -657,28 +657,36 @@ __global__ void __launch_bounds__(kBlock) newton_kernel(const __grid_constant__ 
         // mixed: cells to be solved again in FP64 wait in a queue of the block
         // until there is one for every thread, so that FP64 iterations run in
         // full warps (as in newton_fp64_queued): 300007 scattered cells 289 ->
-        // 203 us, with the bookkeeping above
+        // 203 us, with the bookkeeping above.  Their outputs are not written
+        // before: the result may lie over an input.
         __shared__ int q_n;
         constexpr int kQ = kMixed ? 2 * kBlock : 1;
         __shared__ int64_t q_i[kQ];
-        __shared__ float q_h[kQ], q_l[kQ];   // the start, a two-float T
-        __shared__ int q_it[kQ];
+        __shared__ float q_h[kQ], q_l[kQ];   // the FP32 iteration's T, two floats
+        __shared__ int q_st[kQ];             // its status (low byte) and iterations
         if (kMixed && threadIdx.x == 0) q_n = 0;
         if (kMixed) __syncthreads();
         auto finish = [&](int e) {
             if constexpr (kMixed) {
                 const int64_t i = q_i[e];
+                float Tres = q_h[e];   // stands where FP64 refuses the mass fractions
+                int st = q_st[e] & 255, it = q_st[e] >> 8;
                 Comp<double, NS> c64;
                 if (comp_fp64_of_fp32<NS>(c64, a.Y, a.ldY, i, a.N, s64[0].sp)) {
+                    // from the FP32 root, or the guess
+                    const double T0 = st == kOk ? (double)Tres + (double)q_l[e]
+                                                : fmin(fmax((double)__ldg(a.Tg + i), kTLo), kTHi);
                     double T64, cp64;
                     int it64;
-                    const int st = newton_solve<double, double, NS, KIJ>(
-                        c64, (double)__ldg(a.hstar + i), (double)__ldg(a.p + i), (double)q_h[e] + (double)q_l[e],
-                        s64[0].sp, s64[0].kij, a.tmid_u, a.max_iter, a.rtol, 1e-6, T64, it64, cp64);
-                    a.Tout[i] = (float)T64;   // over the FP32 result
-                    a.status[i] = st;
-                    if (a.iters) a.iters[i] = q_it[e] + it64;
+                    st = newton_solve<double, double, NS, KIJ>(c64, (double)__ldg(a.hstar + i), (double)__ldg(a.p + i),
+                                                               T0, s64[0].sp, s64[0].kij, a.tmid_u, a.max_iter, a.rtol,
+                                                               1e-6, T64, it64, cp64);
+                    Tres = (float)T64;
+                    it += it64;
                 }
+                a.Tout[i] = Tres;
+                a.status[i] = st;
+                if (a.iters) a.iters[i] = it;
             }
         };
         // FP32 thermodynamics resolve h to ~1e-7 of its scale: floor the tolerance
@@ -691,6 +699,7 @@ __global__ void __launch_bounds__(kBlock) newton_kernel(const __grid_constant__ 
                 bool ok = load_comp<float, NS>(c, a.Y, a.ldY, i, a.N, sp);
                 ok = ok && isfinite(hs) && isfinite(Tg) && (p > 0.f) && isfinite(p);
                 int st = kBadInput, it = 0;
+                bool queued = false;
                 Temp2 Tres = {__int_as_float(0x7fc00000), 0.f};
                 if (ok) {
                     const float T0 = fminf(fmaxf(Tg, (float)kTLo), (float)kTHi);
@@ -699,19 +708,22 @@ __global__ void __launch_bounds__(kBlock) newton_kernel(const __grid_constant__ 
                                                        jump_tol, Tres, it, cp_last);
                     if constexpr (kMixed) {
                         // FP64 where FP32 is least reliable: failed cells, and cells in
-                        // the pseudo-boiling band, from the FP32 root (or the guess)
+                        // the pseudo-boiling band
                         if (st != kOk || cp_last > (float)kPseudoCriticalCp * cp_ideal_mass<float, NS>(c, Tres.h, sp)) {
                             const int e = atomicAdd(&q_n, 1);
                             q_i[e] = i;
-                            q_h[e] = st == kOk ? Tres.h : T0;
-                            q_l[e] = st == kOk ? Tres.l : 0.f;
-                            q_it[e] = it;
+                            q_h[e] = Tres.h;
+                            q_l[e] = Tres.l;
+                            q_st[e] = st | it << 8;
+                            queued = true;
                         }
                     }
                 }
-                a.Tout[i] = Tres.h;
-                a.status[i] = st;
-                if (a.iters) a.iters[i] = it;
+                if (!queued) {
+                    a.Tout[i] = Tres.h;
+                    a.status[i] = st;
+                    if (a.iters) a.iters[i] = it;
+                }
             }
             if constexpr (kMixed) queue_round(&q_n, (int)threadIdx.x, (int)blockDim.x, finish);
         }
