@@ -276,6 +276,66 @@ __global__ void __launch_bounds__(kSpBlock, 6) species_fix_kernel(const __grid_c
             }
             continue;
         }
+        if (a.Dk && !prs::fix_range(T)) {
+            const double inv_s = M<double>::rcp(s);
+            double x[9], D[9];
+#pragma unroll
+            for (int k = 0; k < 9; ++k) x[k] = s_x[k][tid] * inv_s;
+            diffusion_general9(y, x, ysum, T, p, N, a.dtab, a.corr, 0, 0, D);
+            for (int k = 0; k < N; ++k) a.Dk[(int64_t)k * a.ldo + i] = D[k];
+        } else if (a.Dk) {
+            // s T^(3/2) / (p sum_j y_j)
+            const double scale = M<double>::div(s * T * M<double>::sqrt(T), p * ysum);
+            const uint64_t bT = i64::bits(T);
+            const uint64_t Tf = i64::signif(bT) >> (1035u - (uint32_t)(bT >> 52));
+            const uint64_t TB = m64::pow_frac_fixed(bT, (uint64_t)(prs::kNB * 18446744073709551616.0));
+            // in loops: unrolled, their ~6000 instructions miss the instruction
+            // cache (the accumulators then live in shared memory)
+#pragma unroll 1
+            for (int u = 0; u < t.n_om; ++u) {
+                const uint64_t om = prs::omega_fix(t.om[u], Tf, TB, s_exp2);
+#pragma unroll 1
+                for (int q = t.first[u]; q < t.first[u + 1]; ++q) {
+                    const double w = prs::pair_fix(t.pair[q], om);
+                    const int k = t.pair[q].k, j = t.pair[q].j;
+                    s_acc[k][tid] = fma(s_x[j][tid], w, s_acc[k][tid]);
+                    s_acc[j][tid] = fma(s_x[k][tid], w, s_acc[j][tid]);
+                }
+            }
+            // (y read again: held across the pairs it would cost 18 registers)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) y[k] = (k < N) ? __ldg(a.Y + (int64_t)k * a.ldY + i) : 0.0;
+            // sum_{j != k} y_j from prefix and suffix sums
+            double others[9];
+            double run = 0;
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                others[k] = run;
+                run += y[k];
+            }
+            run = 0;
+#pragma unroll
+            for (int k = 8; k >= 0; --k) {
+                others[k] += run;
+                run += y[k];
+            }
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                if (k >= N) break;
+                const double acc = s_acc[k][tid];
+                double D;
+                if (acc > 0.0) {
+                    D = M<double>::div(others[k] * scale, acc);
+                } else {   // alone in the cell: self-diffusion, the general form
+                    const double *ie = a.dtab + 18, *epsB = ie + 81, *ic = epsB + 81;
+                    const double TmB = prk::pow_neg<double>(T, prs::kNB);
+                    D = M<double>::div(M<double>::div(T * M<double>::sqrt(T), p),
+                                       prs::omega_d<double>(T * ie[10 * k], TmB * epsB[10 * k]) * ic[10 * k]);
+                }
+                a.Dk[(int64_t)k * a.ldo + i] = D;
+            }
+        }
+        // (last: hk may lie over Y, which is read again above)
         if (a.hk) {
             const double iT = M<double>::rcp(T);
 #pragma unroll 1
@@ -285,66 +345,6 @@ __global__ void __launch_bounds__(kSpBlock, 6) species_fix_kernel(const __grid_c
                 const double h = fma(fma(fma(fma(e[4], T, e[3]), T, e[2]), T, e[1]), T, e[0]);
                 a.hk[(int64_t)k * a.ldo + i] = fma(e[5], iT, h);
             }
-        }
-        if (!a.Dk) continue;
-        if (!prs::fix_range(T)) {
-            const double inv_s = M<double>::rcp(s);
-            double x[9], D[9];
-#pragma unroll
-            for (int k = 0; k < 9; ++k) x[k] = s_x[k][tid] * inv_s;
-            diffusion_general9(y, x, ysum, T, p, N, a.dtab, a.corr, 0, 0, D);
-            for (int k = 0; k < N; ++k) a.Dk[(int64_t)k * a.ldo + i] = D[k];
-            continue;
-        }
-        // s T^(3/2) / (p sum_j y_j)
-        const double scale = M<double>::div(s * T * M<double>::sqrt(T), p * ysum);
-        const uint64_t bT = i64::bits(T);
-        const uint64_t Tf = i64::signif(bT) >> (1035u - (uint32_t)(bT >> 52));
-        const uint64_t TB = m64::pow_frac_fixed(bT, (uint64_t)(prs::kNB * 18446744073709551616.0));
-        // in loops: unrolled, their ~6000 instructions miss the instruction
-        // cache (the accumulators then live in shared memory)
-#pragma unroll 1
-        for (int u = 0; u < t.n_om; ++u) {
-            const uint64_t om = prs::omega_fix(t.om[u], Tf, TB, s_exp2);
-#pragma unroll 1
-            for (int q = t.first[u]; q < t.first[u + 1]; ++q) {
-                const double w = prs::pair_fix(t.pair[q], om);
-                const int k = t.pair[q].k, j = t.pair[q].j;
-                s_acc[k][tid] = fma(s_x[j][tid], w, s_acc[k][tid]);
-                s_acc[j][tid] = fma(s_x[k][tid], w, s_acc[j][tid]);
-            }
-        }
-        // (y read again: held across the pairs it would cost 18 registers)
-#pragma unroll
-        for (int k = 0; k < 9; ++k) y[k] = (k < N) ? __ldg(a.Y + (int64_t)k * a.ldY + i) : 0.0;
-        // sum_{j != k} y_j from prefix and suffix sums
-        double others[9];
-        double run = 0;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            others[k] = run;
-            run += y[k];
-        }
-        run = 0;
-#pragma unroll
-        for (int k = 8; k >= 0; --k) {
-            others[k] += run;
-            run += y[k];
-        }
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            if (k >= N) break;
-            const double acc = s_acc[k][tid];
-            double D;
-            if (acc > 0.0) {
-                D = M<double>::div(others[k] * scale, acc);
-            } else {   // alone in the cell: self-diffusion, the general form
-                const double *ie = a.dtab + 18, *epsB = ie + 81, *ic = epsB + 81;
-                const double TmB = prk::pow_neg<double>(T, prs::kNB);
-                D = M<double>::div(M<double>::div(T * M<double>::sqrt(T), p),
-                                   prs::omega_d<double>(T * ie[10 * k], TmB * epsB[10 * k]) * ic[10 * k]);
-            }
-            a.Dk[(int64_t)k * a.ldo + i] = D;
         }
     }
 }
