@@ -22,6 +22,7 @@
 // form (pr_device.cuh).
 #pragma once
 
+#include "pr_cubic.cuh"
 #include "pr_kernels.cuh"
 
 namespace prk {
@@ -126,69 +127,13 @@ __device__ __forceinline__ int fix9_comp(const Fix9 &t, const double (&y)[9], Fi
     return kFixOk;
 }
 
-// Conversions on the integer pipe (truncating; magnitudes below FP32's normal
-// range become 0): for residuals and derivatives, whose last bits do not matter.
-__device__ __forceinline__ float float_of(double x)
-{
-    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-    const uint32_t e = (hi >> 20) & 0x7FFu;
-    const uint32_t m = ((hi & 0x000FFFFFu) << 3) | (lo >> 29);
-    return __uint_as_float((hi & 0x80000000u) | (e > 896u ? ((e - 896u) << 23) | m : 0u));
-}
-__device__ __forceinline__ double double_of(float x)   // exact for normal x and 0
-{
-    const uint32_t b = __float_as_uint(x);
-    const uint32_t hi = (b & 0x80000000u) | ((b & 0x7F800000u) ? ((b & 0x7FFFFFFFu) >> 3) + 0x38000000u : 0u);
-    return __hiloint2double((int)hi, (int)(b << 29));
-}
-
-// Newton's polish of a cubic's root, the residual in FP64, its quotient by the
-// derivative in FP32: the quotient's relative error of 1e-7 shortens the next
-// step by as much, the limit is the FP64 residual's alone.
-__device__ __forceinline__ double cubic_polish_mixed(double z, double c2, double c1, double c0)
-{
-    const float c22f = 2.f * float_of(c2), c1f = float_of(c1);
-#pragma unroll 1
-    for (int it = 0; it < 12; ++it) {
-        const double f = fma(fma(z + c2, z, c1), z, c0);
-        const float zf = float_of(z), d = fmaf(fmaf(3.f, zf, c22f), zf, c1f);
-        if (d == 0.f) break;
-        const float dz = __fdividef(float_of(f), d);
-        z -= double_of(dz);
-        if (fabsf(dz) <= 4.44e-16f * fabsf(zf)) break;
-    }
-    return z;
-}
-
 // The physical root, as cubic_phys_roots and select_root: the common case of
-// one seed above B directly, the others through them.  Returns the status.
+// one root above B directly, the others through them.  Returns the status.
 __device__ __forceinline__ int cubic_root_fix(double c2, double c1, double c0, double A, double B, double &Z, int &nroots)
 {
-    const double c23 = c2 * (1.0 / 3.0);
-    const double P = fma(-c2, c23, c1), Q = fma(c23, fma(2.0 * c23, c23, -c1), c0);
-    const float Pf = float_of(P), Qf = float_of(Q), c23f = float_of(c23);
-    const float hq = 0.5f * Qf, tp = Pf * (1.f / 3.f), t3 = tp * tp * tp, h2 = hq * hq, disc = h2 + t3;
-    const float Bcut = float_of(B) * (1.f - 1e-3f);
-    float seed = 0.f;
-    bool one = false;   // exactly one seed above B
-    if (fabsf(disc) > 1e-4f * (h2 + fabsf(t3))) {   // the sign of the discriminant is settled
-        if (disc > 0.f) {
-            const float u = cbrtf(-hq - copysignf(sqrtf(disc), hq));
-            seed = ((u != 0.f) ? (u - Pf / (3.f * u)) : 0.f) - c23f;
-            one = seed > Bcut;
-        } else {
-            const float m = 2.f * sqrtf(fmaxf(-tp, 0.f));
-            float arg = (m > 0.f) ? (3.f * Qf) / (Pf * m) : 0.f;
-            arg = fminf(1.f, fmaxf(-1.f, arg));
-            const float th = acosf(arg) * (1.f / 3.f);
-            seed = m * cosf(th) - c23f;   // the largest; the middle one below B settles the smallest
-            one = seed > Bcut && !(m * cosf(th + 4.18879020478639f) - c23f > Bcut);
-        }
-    }
-    if (one) {
-        Z = cubic_polish_mixed(double_of(seed), c2, c1, c0);
+    if (cubic_single_root(c2, c1, c0, B, Z)) {
         nroots = 1;
-        if (Z > B) return kOk;
+        return kOk;
     }
     double zr[3];
     nroots = cubic_phys_roots<double>(c2, c1, c0, B, zr);
