@@ -216,6 +216,34 @@ bool fill_fix9(Fix9 &t, const HostTable &h, int N, int flags, bool has_kij, doub
         t.en[r] = to_mac31(w5, 5 * N, o5);
     }
     t.ea6 = to_mac31(w6, 18, o6);
+    // A sum is off by up to 12 units of 2^-58 of its largest constant, whichever
+    // species the cell holds.  The constants of each species alone, and the
+    // moles of one, may be smaller than the table's largest by what still leaves
+    // 12 x 2^-52 of the sum (moles 2^-53; a_6, a temperature, 1.5e-12 K), two
+    // decades under the 1e-12 of the accepted step; else the general form.  The
+    // nine species of the flame: b 2^0.7, u 2^4.3, NASA-7 2^5.3 (methane's range
+    // above the switch against hydrogen atoms'), a_6 2^14.3, moles 2^5.5.
+    ld top_b = 0, top_u0 = 0, top_u1 = 0, top_n[2] = {0, 0}, top_6 = 0;
+    ld own_n[2][9] = {};
+    for (int k = 0; k < N; ++k) {
+        top_b = fmaxl(top_b, Ob * Rg * (ld)h.Tc[k] / (ld)h.pc[k]);
+        top_u0 = fmaxl(top_u0, g[k] * (1.0L + kap[k]));
+        top_u1 = fmaxl(top_u1, fabsl(g[k] * kq[k]));
+        for (int r = 0; r < 2; ++r) {
+            const double *a = r ? h.nasa_hi[k] : h.nasa_lo[k];
+            ld f = 1.0L;
+            for (int j = 0; j < 5; ++j, f *= r ? 4096.0L : 1024.0L) own_n[r][k] = fmaxl(own_n[r][k], fabsl(f * (ld)a[j]));
+            top_n[r] = fmaxl(top_n[r], own_n[r][k]);
+            top_6 = fmaxl(top_6, fabsl((ld)a[5]));
+        }
+    }
+    for (int k = 0; k < N; ++k) {
+        const ld b = Ob * Rg * (ld)h.Tc[k] / (ld)h.pc[k], iW = 1.0L / ((ld)h.W[k] * 1e-3L);
+        if (!(iWmax <= 512.0L * iW && top_b <= 64.0L * b)) return false;
+        if (!(top_u0 + 64.0L * top_u1 <= 64.0L * g[k] * (1.0L + kap[k]))) return false;   // (sqrt T below 64)
+        for (int r = 0; r < 2; ++r)
+            if (!(top_n[r] <= 64.0L * own_n[r][k] && top_6 <= 32768.0L * own_n[r][k])) return false;
+    }
     // every unit within a normal double's exponents
     for (int e : {t.eb, t.eu0, t.eu1, t.en[0], t.en[1], t.ea6})
         if (e < -800 || e > 800) return false;
