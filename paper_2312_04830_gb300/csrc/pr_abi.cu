@@ -244,6 +244,12 @@ bool fill_fix9(Fix9 &t, const HostTable &h, int N, int flags, bool has_kij, doub
         for (int r = 0; r < 2; ++r)
             if (!(top_n[r] <= 64.0L * own_n[r][k] && top_6 <= 32768.0L * own_n[r][k])) return false;
     }
+    ld wW[9], wb[9];
+    for (int k = 0; k < N; ++k) {
+        wW[k] = 1.0L / ((ld)h.W[k] * 1e-3L);
+        wb[k] = Ob * Rg * (ld)h.Tc[k] / (ld)h.pc[k];
+    }
+    if (!fill_warm(t.warm, wW, wb, N)) return false;
     // every unit within a normal double's exponents
     for (int e : {t.eb, t.eu0, t.eu1, t.en[0], t.en[1], t.ea6})
         if (e < -800 || e > 800) return false;

@@ -24,6 +24,7 @@
 
 #include "pr_cubic.cuh"
 #include "pr_kernels.cuh"
+#include "pr_warm.cuh"
 
 namespace prk {
 
@@ -40,6 +41,7 @@ struct Fix9Rec {
 };
 struct Fix9 {
     Fix9Rec sp[9];
+    WarmTab warm;
     int32_t eb, eu0, eu1, en[2], ea6;   // a sum's unit is 2^e
     double iWmax;               // max(1/W) [mol/kg]
     double rWmax;               // its inverse

@@ -26,28 +26,19 @@ static __device__ __noinline__ void newton_finish9(const NewtonArgs<double> &a, 
 // into Tout and the FP32 cp at it, as bits, into the status array (0 where
 // the warm start failed: T is then the clamped guess; -1: a guess refused) ...
 __global__ void __launch_bounds__(kBlock) newton_warm_kernel(const __grid_constant__ NewtonArgs<double> a,
-                                                             const __grid_constant__ ParamTab<float, 9, false> t)
+                                                             const __grid_constant__ ParamTab<float, 9, false> t,
+                                                             const __grid_constant__ WarmTab w)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += stride) {
         const float hs = (float)__ldg(a.hstar + i), p = (float)__ldg(a.p + i);
         const double Tg = a.Tg[i];   // Tg may be Tout
         const double T0 = fmin(fmax(Tg, kTLo), kTHi);
+        double y[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) y[k] = (k < a.N) ? __ldg(a.Y + (int64_t)k * a.ldY + i) : 0.0;
         Comp<float, 9> c;
-        float s = 0.f, bm = 0.f;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            c.x[k] = (k < a.N) ? (float)__ldg(a.Y + (int64_t)k * a.ldY + i) * t.sp[k].inv_W : 0.f;
-            s += c.x[k];
-        }
-        const float is = 1.f / s;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            c.x[k] *= is;
-            bm = fmaf(c.x[k], t.sp[k].b, bm);
-        }
-        c.Wbar = is;
-        c.bm = bm;
+        warm_comp(w, y, c);
         // warm_start_fp32's iteration with its evaluations at one place, in
         // line, the tables as constant operands (states refused by the second
         // launch pass through here too: the loop is bounded)
@@ -146,21 +137,11 @@ __global__ void __launch_bounds__(kBlock, 4) newton_fix_kernel(const __grid_cons
                 newton_fix_cell(a, t, i, a.Tout[i], cp32, s32.sp, &q_n, q_i, q_T, q_h, q_cp, q_first, cp32 >= 0.f);
             } else {
                 const double Tg = __ldg(a.Tg + i);
+                double y[9];
+#pragma unroll
+                for (int k = 0; k < 9; ++k) y[k] = (k < a.N) ? __ldg(a.Y + (int64_t)k * a.ldY + i) : 0.0;
                 Comp<float, 9> cf;
-                float s = 0.f, bm = 0.f;
-#pragma unroll
-                for (int k = 0; k < 9; ++k) {
-                    cf.x[k] = (k < a.N) ? (float)__ldg(a.Y + (int64_t)k * a.ldY + i) * s32.sp[k].inv_W : 0.f;
-                    s += cf.x[k];
-                }
-                const float is = 1.f / s;
-#pragma unroll
-                for (int k = 0; k < 9; ++k) {
-                    cf.x[k] *= is;
-                    bm = fmaf(cf.x[k], s32.sp[k].b, bm);
-                }
-                cf.Wbar = is;
-                cf.bm = bm;
+                warm_comp(t.warm, y, cf);
                 bool wok;
                 float cp32;
                 const double T = warm_start_fp32<9, false>(cf, fmin(fmax(Tg, kTLo), kTHi), __ldg(a.hstar + i),
@@ -195,7 +176,7 @@ void launch_newton_fix(const NewtonArgs<double> &a, const Fix9 &t, const void *h
     // (65536 cells, in one wave: 69 us against 72; 131072: 114 against 88;
     // 2.1 M cells: 1238 against 683)
     if (a.n > (int64_t)occ[2] * sms * kBlock && own) {
-        newton_warm_kernel<<<grid_for(a.n, occ[0], sms), kBlock, 0, st>>>(a, make_tab<float, 9, false>(htab32));
+        newton_warm_kernel<<<grid_for(a.n, occ[0], sms), kBlock, 0, st>>>(a, make_tab<float, 9, false>(htab32), t.warm);
         newton_fix_kernel<true><<<grid_for(a.n, occ[1], sms), kBlock, 0, st>>>(a, t);
     } else {
         const int b = block_for(a.n, sms);

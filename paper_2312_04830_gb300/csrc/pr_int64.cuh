@@ -136,6 +136,41 @@ I64_FN float approx_rsqrt(float x)
 #endif
 }
 
+// 32-bit operations: a >> s (0 from s = 32 on), the high word of a << s for s
+// < 32, leading zeros of a nonzero a, a as a float to nearest
+I64_FN uint32_t shr32(uint32_t a, uint32_t s)
+{
+#ifdef __CUDACC__
+    return __funnelshift_rc(a, 0u, s);
+#else
+    return s < 32 ? a >> s : 0;
+#endif
+}
+I64_FN uint32_t shl_hi32(uint64_t a, uint32_t s)
+{
+#ifdef __CUDACC__
+    return __funnelshift_l(lo32(a), hi32(a), s);
+#else
+    return hi32(a << s);
+#endif
+}
+I64_FN uint32_t clz32(uint32_t a)
+{
+#ifdef __CUDACC__
+    return (uint32_t)__clz((int)a);
+#else
+    return (uint32_t)__builtin_clz(a);
+#endif
+}
+I64_FN float to_float(uint32_t a)
+{
+#ifdef __CUDACC__
+    return __uint2float_rn(a);
+#else
+    return (float)a;
+#endif
+}
+
 // biased exponent field; significand of a normal number, its leading 1 at bit 63
 I64_FN uint32_t expo(uint64_t b) { return (uint32_t)(b >> 52) & 0x7FFu; }
 I64_FN uint64_t signif(uint64_t b) { return (b << 11) | 0x8000000000000000ull; }
