@@ -16,6 +16,7 @@
 
 #include "pr_device.cuh"
 #include "pr_queue.cuh"
+#include "pr_two.cuh"
 
 namespace prk {
 
@@ -375,20 +376,6 @@ __device__ __forceinline__ int newton_solve(const Comp<Real, NS> &c, double hs, 
     return st;
 }
 
-// A temperature as an unevaluated sum of two floats, h = the sum rounded.
-struct Temp2 {
-    float h, l;
-};
-__device__ __forceinline__ Temp2 temp2_add(Temp2 a, float b)
-{
-    // two-sum of h and b (Knuth), the tail added and the result renormalised
-    const float s = __fadd_rn(a.h, b), bb = __fsub_rn(s, a.h);
-    const float e = __fadd_rn(__fadd_rn(__fsub_rn(a.h, __fsub_rn(s, bb)), __fsub_rn(b, bb)), a.l);
-    const float h = __fadd_rn(s, e);
-    return {h, __fsub_rn(e, __fsub_rn(h, s))};
-}
-__device__ __forceinline__ bool temp2_less(Temp2 a, Temp2 b) { return a.h < b.h || (a.h == b.h && a.l < b.l); }
-
 // newton_solve for the FP32 and mixed inversions, its bookkeeping in FP32: T
 // as a two-float number (48 bits; h(T) is evaluated at its rounded value
 // anyway), the residual h - h* of two FP32 numbers, the step's quotient and
@@ -464,9 +451,9 @@ __device__ __forceinline__ int newton_solve_f32(const Comp<float, NS> &c, float 
     return st;
 }
 
-// Mass-specific ideal-gas cp of a cell [J/(kg K)] (NASA-7).
+// Molar ideal-gas cp of a cell [J/(mol K)] (NASA-7).
 template <typename Real, int NS>
-__device__ __forceinline__ Real cp_ideal_mass(const Comp<Real, NS> &c, Real T, const SpeciesRec<Real> *sp)
+__device__ __forceinline__ Real cp_ideal_molar(const Comp<Real, NS> &c, Real T, const SpeciesRec<Real> *sp)
 {
     Real s = 0;
 #pragma unroll
@@ -475,7 +462,7 @@ __device__ __forceinline__ Real cp_ideal_mass(const Comp<Real, NS> &c, Real T, c
         const Real cpk = M<Real>::fma(M<Real>::fma(M<Real>::fma(M<Real>::fma(a[4], T, a[3]), T, a[2]), T, a[1]), T, a[0]);
         s = M<Real>::fma(c.x[k], cpk, s);
     }
-    return M<Real>::div(s, c.Wbar);
+    return s;
 }
 
 // Composition in FP64 from FP32 mass fractions (the FP64 re-solve of the
@@ -709,7 +696,8 @@ __global__ void __launch_bounds__(kBlock) newton_kernel(const __grid_constant__ 
                     if constexpr (kMixed) {
                         // FP64 where FP32 is least reliable: failed cells, and cells in
                         // the pseudo-boiling band
-                        if (st != kOk || cp_last > (float)kPseudoCriticalCp * cp_ideal_mass<float, NS>(c, Tres.h, sp)) {
+                        if (st != kOk ||
+                            product_less((float)kPseudoCriticalCp, cp_ideal_molar<float, NS>(c, Tres.h, sp), cp_last, c.Wbar)) {
                             const int e = atomicAdd(&q_n, 1);
                             q_i[e] = i;
                             q_h[e] = Tres.h;
