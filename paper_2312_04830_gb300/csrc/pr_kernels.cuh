@@ -721,11 +721,17 @@ __global__ void __launch_bounds__(kBlock) newton_kernel(const __grid_constant__ 
 
 
 // ------------------------------------------------------------- launchers
-// Threads per block: one warp while that gives every block an SM of its own,
-// then two.  A small call is as long as its busiest SM, whose FP64 pipe takes
-// 16 cycles per warp instruction: 1000 cells of FP64 properties 43.7 -> 41.7 us
-// a call, most of it one cell's dependent chain (38 us in the kernel with one
-// warp an SM, 41 with two, 44 with four).
+// Threads per block of the FP64 properties and of every inversion: one warp
+// while that gives every block an SM of its own, then two.  A small call is as
+// long as its busiest SM, whose FP64 pipe (in the mixed inversion, of its
+// re-solved cells) takes 16 cycles per warp instruction.  Device time in a
+// replayed graph, us, small blocks | whole ones: FP64 properties of 100, 1000,
+// 4000, 9728 cells 37.7 | 39.5, 38.7 | 39.4, 42.4 | 43.8, 41.9 | 43.5 (500: 40.0
+// | 39.7), FP64 inversion 53.2 | 59.6, 58.8 | 59.5, 179 | 182, 247 | 250, mixed
+// inversion of 100, 1000, 2000, 7000 cells 8.5 | 7.8, 37.0 | 36.4, 102 | 115, 125
+// | 127, FP32 inversion within 2 % either way; most of a call is one cell's
+// dependent chain.  FP32 and mixed properties take whole blocks: 2000 cells 4.25
+// | 4.21 and 7.9 | 7.6, 4864 cells 4.6 | 4.3 and 15.6 | 15.0.
 inline int block_for(int64_t n, int sms) { return n <= 32 * (int64_t)sms ? 32 : n <= 64 * (int64_t)sms ? 64 : kBlock; }
 
 inline int grid_for(int64_t n, int occ, int sms, int block = kBlock)
@@ -739,7 +745,7 @@ inline int grid_for(int64_t n, int occ, int sms, int block = kBlock)
 template <typename Real, typename RZ, int NS>
 void launch_props(const PropsArgs<Real> &a, const void *htab, bool kij, int occ, int sms, cudaStream_t st)
 {
-    const int b = block_for(a.n, sms), g = grid_for(a.n, occ, sms, b);
+    const int b = sizeof(Real) == 8 ? block_for(a.n, sms) : kBlock, g = grid_for(a.n, occ, sms, b);
     if (kij) props_kernel<Real, RZ, NS, true><<<g, b, 0, st>>>(a, make_tab<Real, NS, true>(htab));
     else props_kernel<Real, RZ, NS, false><<<g, b, 0, st>>>(a, make_tab<Real, NS, false>(htab));
 }
