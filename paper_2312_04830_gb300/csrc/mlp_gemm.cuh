@@ -17,8 +17,8 @@
 //
 // Per 65536 x 512 x 512 GEMM of a training step, us, in the step (8 epilogue
 // warps and single CTAs | 16 warps and pairs): hidden layer 48 | 46, input
-// gradient 54 | 50, weight gradient 39 | 33; with K = 64 hidden 34 | 28 and
-// input gradient 48 | 35.  What is left above the MMAs' 15 us: 8 to 10 us to
+// gradient 54 | 50, weight gradient 39 | 33; with K = 64, on single CTAs with
+// 16 warps too, hidden 34 | 27 and input gradient 48 | 32.  What is left above the MMAs' 15 us: 8 to 10 us to
 // launch, fill and drain, and the epilogue's traffic, which slows the main
 // loop (a hidden layer's takes 27 us without an epilogue, 36 without its
 // stores and 42 without the GeLU).
@@ -151,8 +151,7 @@ __device__ __forceinline__ float2 gelu2(float2 a, float2 b)
     return __ffma2_rn(hz, t, hz);
 }
 
-// gelu_and_grad of z = a + b on two lanes at once (packed FP32): the same
-// operations in the same order as the scalar form, so the same bits.
+// GeLU(z) and GeLU'(z) of z = a + b on two lanes at once (packed FP32).
 __device__ __forceinline__ void gelu_and_grad2(float2 a, float2 b, float2 &g, float2 &dg)
 {
     const float2 z = __fadd2_rn(a, b);
@@ -164,16 +163,6 @@ __device__ __forceinline__ void gelu_and_grad2(float2 a, float2 b, float2 &g, fl
     const float2 dk = __ffma2_rn(make_float2(3.0f * kGeluKC, 3.0f * kGeluKC), z2, make_float2(kGeluK, kGeluK));
     const float2 omt = __ffma2_rn(make_float2(-t.x, -t.y), t, make_float2(1.0f, 1.0f));
     dg = __ffma2_rn(__fmul2_rn(hz, omt), dk, __ffma2_rn(make_float2(0.5f, 0.5f), t, make_float2(0.5f, 0.5f)));
-}
-
-__device__ __forceinline__ void gelu_and_grad(float z, float &g, float &dg)
-{
-    const float z2 = z * z;
-    const float t = tanh_approx(z * fmaf(kGeluKC, z2, kGeluK));
-    const float hz = 0.5f * z;
-    g = fmaf(hz, t, hz);
-    const float dk = fmaf(3.0f * kGeluKC, z2, kGeluK);      // d/dz of k (z + c z^3)
-    dg = fmaf(hz * fmaf(-t, t, 1.0f), dk, fmaf(0.5f, t, 0.5f));
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b)

@@ -269,13 +269,16 @@ __global__ void transpose_w_kernel(SgDev d)
     }
 }
 
-// Launch of a kernel of a training step or an inference call: its blocks may take their places (and,
-// in a GEMM, set up barriers and tensor memory) while the kernel before it
-// drains; each waits (pdl_wait) before it touches global memory.  A step is 20
-// launches with 8 to 10 us each to launch, fill and drain: 512 x 4, batch
-// 65536, 600 us a step launched one after the other, 557 so; an inference call
-// of 20011 cells (256 x 3, in a graph) 37.8 us and 34.8.  `cluster` CTAs to a
-// cluster.
+// Launch of a kernel of a training step or an inference call: its blocks may
+// take their places (and, in a GEMM, set up barriers and tensor memory) while
+// the kernel before it drains.  The training kernels wait (pdl_wait) before they
+// touch global memory.  The inference kernels first read what no kernel of the
+// call writes (biases, species and pair tables): prep_infer_kernel starts after
+// everything before it in the stream has ended, so these are complete when the
+// kernel after it starts.  A step is 20 launches with 8 to 10 us each to
+// launch, fill and drain: 512 x 4, batch 65536, 600 us a step launched one after
+// the other, 557 so; an inference call of 20011 cells (256 x 3, in a graph) 37.8
+// us and 34.8.  `cluster` CTAs to a cluster.
 template <class... P, class... A>
 cudaError_t launch_step(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, int cluster, cudaStream_t st,
                         const A &...args)
@@ -1654,6 +1657,7 @@ pr_status surrogate_infer(sg_model *m, int64_t n, const float *T, const float *p
         const int mt = ceil_div(mc, 128);
         PR_CUDA_TRY(cudaMemsetAsync(m->d_count, 0, 4, st));
         const int pb = ceil_div(mc, 256);
+        // in stream order, not by launch_step: the kernels after it rely on it
         prep_infer_kernel<<<pb < 4096 ? pb : 4096, 256, 0, st>>>(d, r0, mc, T, p, Y, ldY, used_fallback,
                                                                  m->d_flags, m->d_list, m->d_count);
         PR_CUDA_TRY(cudaGetLastError());

@@ -22,8 +22,10 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p)
 // A kernel launched with programmatic stream serialisation may start once
 // every block of its predecessor has called pdl_release (or has ended); past
 // pdl_wait the predecessor has ended and what it wrote is visible.  Every
-// thread of such a kernel that touches global memory waits first, so a kernel
-// that has ended had all its predecessors end before it.
+// thread of such a kernel waits, so a kernel that has ended had all its
+// predecessors end before it.  Before the wait it may read only what was
+// complete when its predecessor started: data that neither the predecessor nor
+// a kernel the predecessor had not itself waited for writes.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
