@@ -17,8 +17,8 @@
 // TOMS 15 (1989) 144 and 16 (1990) 378).  Every intermediate is unsigned: the
 // seeds are taken below the true value, so that residuals are positive.
 // Errors against 60-digit references before the final rounding: rcp 2^-61.5,
-// rsqrt 2^-60, relative; exp2 2^-60.4, log2 2^-60.7, absolute: the rounded
-// results are within 0.51 units in the last place.
+// rsqrt 2^-60, relative; exp2 2^-60.4, log2 2^-60.7, absolute.  (Rounded: see
+// pr_math64.cuh.)
 //
 // Measured rates (per clock and SM): wide 32 x 32-bit multiply-adds 28, 64-bit
 // high products 7.5, DFMA 1.7-2.  A division (~45 instructions, 5 wide

@@ -1,8 +1,7 @@
 // FP64 elementary functions of the property paths.  The FP64 pipe is their
 // scarce unit (2 operations per clock per SM on GB300), so the usual argument
-// ranges are computed on the integer pipe (pr_int64.cuh, at most 0.6 units in
-// the last place before any range restriction below); what they leave goes to
-// the forms here, or to CUDA's functions:
+// ranges are computed on the integer pipe (pr_int64.cuh); what they leave goes
+// to the forms here, or to CUDA's functions:
 //   rcp, div, sqrt   normal operands and results;
 //   exp              |x| < 64 (else CUDA's exp);
 //   expm1            2^-7 <= |x| < 64 (smaller: Tang's form below);
@@ -17,8 +16,12 @@
 // log: F = 1 + j/128 nearest the significand m: ln x = e ln2 + ln F + ln(1 + r),
 // r = (m - F)/F (m - F exact; 1/F from a table and one correction step),
 // ln(1 + r) by its Taylor polynomial to r^8 (|r| <= 1/256).
-// Errors on the tested ranges (tests/test_gpu_math64.py, extended-precision
-// references): within 1.5 ulp.
+// Errors in units in the last place: rcp, div and sqrt within 0.51 (2^-60 before
+// the rounding); against quad precision, 2 M arguments a range: exp 0.59 (the
+// argument's 64 bits at |x| near 64; 0.51 below 1), log and log1p 0.60 in the
+// integer form (1.2 and 1.5 in Tang's near zero), expm1 0.64 from 2^-5, 1.08
+// from 2^-7 to 2^-5 (the absolute error of 2^-60 against a small result), 1.35
+// below.  Tests (tests/test_gpu_math64.py): within 1.5.
 #pragma once
 
 #include <cuda_runtime.h>
