@@ -271,7 +271,8 @@ __device__ __forceinline__ bool one_step_ok(const FirstEval &f, double T, double
     return clear;
 }
 
-// h(T) and cp(T) in FP32 with FP32 arguments (the warm start's evaluations).
+// h(T) and cp(T) in FP32 with FP32 arguments (the warm start's evaluations, and
+// the FP32 inversion's of more than 9 species).
 template <int NS, bool KIJ>
 __device__ __noinline__ int eval_h_f32(const Comp<float, NS> &c, float T, float p, const SpeciesRec<float> *sp,
                                        const float *kij, float tmid_u, float &h, float &cp)
@@ -384,7 +385,10 @@ __device__ __forceinline__ int newton_solve(const Comp<Real, NS> &c, double hs, 
 // 44 %: 4.5 M cells of the flame field 703 us (535 us with the division on
 // the integer pipe), 365 us with this bookkeeping, and 326 us with the
 // thermodynamics in line at one place and the tables in the parameter space
-// (35.5 M of 336 M instructions were loads of tables and arguments).
+// (35.5 M of 336 M instructions were loads of tables and arguments).  With 32
+// species in line the FP32 kernel takes 255 registers and spills: out of line
+// there (200000 cells of 14 species 126 us in line, 78 out of line; mixed 350 and
+// 360, in line).
 template <typename RZ, int NS, bool KIJ>
 __device__ __forceinline__ int newton_solve_f32(const Comp<float, NS> &c, float hs, float p, float T0,
                                                 const SpeciesRec<float> *sp, const float *kij, float tmid_u,
@@ -403,16 +407,24 @@ __device__ __forceinline__ int newton_solve_f32(const Comp<float, NS> &c, float 
     int phase = 0;
 #pragma unroll 1
     while (true) {
-        Thermo<float> th;
-        thermo<float, RZ, NS, KIJ>(c, Te, p, sp, kij, th, tmid_u);
-        const float h = th.h, cp = th.cp;
+        float h = 0.f, cp = 0.f;
+        bool none;
+        if constexpr (NS > 9 && sizeof(RZ) == 4) {
+            none = eval_h_f32<NS, KIJ>(c, Te, p, sp, kij, tmid_u, h, cp) != 0;
+        } else {
+            Thermo<float> th;
+            thermo<float, RZ, NS, KIJ>(c, Te, p, sp, kij, th, tmid_u);
+            none = th.status == kNoRoot;
+            h = th.h;
+            cp = th.cp;
+        }
         if (phase == 2) {
-            if (th.status == kNoRoot) { st = kNoRoot; break; }
+            if (none) { st = kNoRoot; break; }
             cp_last = cp;
             st = (fabsf(h - hs) <= jump_tol * fmaxf(fabsf(hs), fabsf(cp) * tn.h)) ? kOk : kHRange;
             break;
         }
-        if (th.status == kNoRoot) { st = kNoRoot; Tres = t; break; }
+        if (none) { st = kNoRoot; Tres = t; break; }
         if (phase == 0) {
             cp_last = cp;
             f = h - hs;
