@@ -4,11 +4,11 @@
 // pair of CTAs) and fused epilogues for every GEMM of the MLP's forward and
 // backward pass.
 //
-// Persistent kernel, one CTA per SM, 18 warps: warp 0 issues TMA loads into
-// an S-stage shared-memory ring, one thread of warp 1 issues the MMAs (K = 16
-// each, 4 per 64-wide k-block), warps 2-17 drain the accumulator and run the
-// epilogue (warp w owns TMEM lane quarter w % 4, i.e. 32 rows, and a quarter
-// of the tile's columns).  The accumulator is double-buffered in TMEM (2 x BN
+// Persistent kernel, one CTA per SM, 18 warps (the plain GEMM 10): warp 0
+// issues TMA loads into an S-stage shared-memory ring, one thread of warp 1
+// issues the MMAs (K = 16 each, 4 per 64-wide k-block), the other warps drain
+// the accumulator and run the epilogue (warp w owns TMEM lane quarter w % 4,
+// i.e. 32 rows, and a quarter, in the plain GEMM a half, of the tile's columns).  The accumulator is double-buffered in TMEM (2 x BN
 // columns), so the epilogue of one tile overlaps the main loop of the next.
 // Tiles are visited with the N index fastest, so the N-tiles of one M-tile run
 // together and share the A tile through L2.  A pair takes two adjacent M-tiles
@@ -84,8 +84,9 @@ struct GemmArgs {
     CUtensorMap tm_out, tm_gd;
 };
 
-constexpr int kEpiWarps = 16;
-constexpr int kThreads = 64 + 32 * kEpiWarps;
+// Epilogue warps: 16, but 8 for the plain GEMM, whose FP32 rows the store units
+// hold (65536 x 512 x 64: 47.5 us with 16, 44.4 with 8; x 512 60.9 and 57.4).
+constexpr int epi_warps(int EPI) { return EPI == kEpiDw ? 8 : 16; }
 
 // Rows of B per TMA box of a K-major GEMM: the half that one CTA of a pair
 // loads (a single CTA loads two boxes, one above the other).
@@ -96,14 +97,17 @@ struct Cfg {
     static constexpr int A_BYTES = BM * BK * 2;
     static constexpr int B_BYTES = (PAIR ? BN / 2 : BN) * BK * 2;
     static constexpr int STAGE = A_BYTES + B_BYTES;
-    static constexpr int COLS = (BN >= 64) ? BN / 4 : BN;   // columns per epilogue warp
+    static constexpr int WARPS = epi_warps(EPI);
+    static constexpr int THREADS = 64 + 32 * WARPS;
+    static constexpr bool SPLIT_N = BN >= 4 * WARPS;                    // each quarter's warps share the columns
+    static constexpr int COLS = SPLIT_N ? BN / (WARPS / 4) : BN;   // columns per epilogue warp
     // output staging, two 2 KB boxes per epilogue warp.  (Without any, the
     // weight gradients have six stages for four: 36 -> 33 us.)
-    static constexpr int STG_BYTES = (EPI == kEpiHidden || EPI == kEpiDx) ? kEpiWarps * 4096 : 0;
+    static constexpr int STG_BYTES = (EPI == kEpiHidden || EPI == kEpiDx) ? WARPS * 4096 : 0;
     static constexpr int S_FIT = (232448 - 1024 - STG_BYTES - 13312) / STAGE;
     static constexpr int S = S_FIT < 8 ? S_FIT : 8;
     static constexpr uint32_t TMEM_COLS = (2 * BN) < 32 ? 32 : 2 * BN;   // two accumulator buffers
-    static constexpr int BAR_BYTES = 8 * (2 * S + 5 + 2 * kEpiWarps) + 24;
+    static constexpr int BAR_BYTES = 8 * (2 * S + 5 + 2 * WARPS) + 24;
     static constexpr int RED_FLOATS = 4 * BN + 16;          // one tile's column sums and loss sums; two tiles' worth
     static constexpr int RED_BYTES = 2 * RED_FLOATS * 4;
     static constexpr int BIAS_BYTES = 1024 * 4;   // bias of up to 1024 output columns
@@ -247,9 +251,10 @@ __device__ __forceinline__ float warp_colsum16(float (&v)[16], int lane)
     return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
+template <int THREADS>
 __device__ __forceinline__ void named_barrier_epi()
 {
-    asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
+    asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
 }
 
 // Tile `t` of the grid-stride walk: K split, M-tile index (of this CTA: a pair
@@ -400,7 +405,7 @@ __device__ __forceinline__ float epilogue_tile(const GemmArgs &a, uint32_t taddr
 }
 
 template <int BN, int EPI, bool PAIR>
-__global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant__ CUtensorMap tmA,
+__global__ void __launch_bounds__(64 + 32 * epi_warps(EPI), 1) gemm_kernel(const __grid_constant__ CUtensorMap tmA,
                                                            const __grid_constant__ CUtensorMap tmB,
                                                            const __grid_constant__ GemmArgs a)
 {
@@ -413,8 +418,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
     uint64_t *acc_full = empty + C::S;     // [2]
     uint64_t *acc_empty = acc_full + 2;    // [2]
     uint64_t *drain = acc_empty + 2;       // (PAIR) every MMA issued has completed
-    uint64_t *gfull = drain + 1;           // [kEpiWarps][2] GeLU'(z) boxes landed
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(gfull + 2 * kEpiWarps);
+    uint64_t *gfull = drain + 1;           // [WARPS][2] GeLU'(z) boxes landed
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(gfull + 2 * C::WARPS);
     float *red = reinterpret_cast<float *>(stg_base + C::STG_BYTES + C::BAR_BYTES);   // 2 x ([4][BN] + 16)
     float *sbias = red + 2 * C::RED_FLOATS;                                          // [N] (N <= 1024)
 
@@ -436,10 +441,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
         }
         for (int b = 0; b < 2; ++b) {
             umma::mbar_init(&acc_full[b], 1);
-            umma::mbar_init(&acc_empty[b], (PAIR ? 2 : 1) * kEpiWarps);
+            umma::mbar_init(&acc_empty[b], (PAIR ? 2 : 1) * C::WARPS);
         }
         umma::mbar_init(drain, 1);
-        for (int b = 0; b < 2 * kEpiWarps; ++b) umma::mbar_init(&gfull[b], 1);
+        for (int b = 0; b < 2 * C::WARPS; ++b) umma::mbar_init(&gfull[b], 1);
         umma::fence_mbar_init();
         umma::tma_prefetch_desc(&tmA);
         umma::tma_prefetch_desc(&tmB);
@@ -485,6 +490,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                     const uint32_t bar =
                         PAIR ? umma::mapa_shared(umma::smem_u32(&full[s]), 0u) : umma::smem_u32(&full[s]);
                     auto load = [&](uint8_t *dst, const CUtensorMap *tm, int c0, int c1) {
+                        if constexpr (EPI == kEpiDw) {
+                            // no policy beside the stores of FP32 rows: with evict_normal on
+                            // the loads 65536 x 512 x 512 takes 66 us, without 57
+                            if constexpr (PAIR) umma::tma_load_2d_pair(dst, tm, bar, c0, c1);
+                            else umma::tma_load_2d(dst, tm, &full[s], c0, c1);
+                            return;
+                        }
                         const uint64_t pol = tm == &tmA ? pol_a : pol_b;
                         if constexpr (PAIR) umma::tma_load_2d_pair_hint(dst, tm, bar, c0, c1, pol);
                         else umma::tma_load_2d_hint(dst, tm, &full[s], c0, c1, pol);
@@ -561,15 +573,15 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
         }
     } else {
         // ------------------------------------------------ epilogue (each CTA)
-        const int ew = warp - 2;                   // 0..15
+        const int ew = warp - 2;
         const int q = warp & 3;                    // TMEM lane quarter this warp may access
-        const int hcol = (BN >= 64) ? (ew >> 2) * C::COLS : 0;   // this warp's first column
-        const bool active = (BN >= 64) || (ew < 4);
+        const int hcol = C::SPLIT_N ? (ew >> 2) * C::COLS : 0;   // this warp's first column
+        const bool active = C::SPLIT_N || (ew < 4);
         const int row = q * 32 + lane;
         uint8_t *stg = stg_base + ew * 4096;
         if (EPI == kEpiHidden || EPI == kEpiOutPhys || EPI == kEpiOutLoss) {
-            for (int col = threadIdx.x - 64; col < a.N; col += 32 * kEpiWarps) sbias[col] = __ldg(a.bias + col);
-            named_barrier_epi();
+            for (int col = threadIdx.x - 64; col < a.N; col += 32 * C::WARPS) sbias[col] = __ldg(a.bias + col);
+            named_barrier_epi<32 * C::WARPS>();
         }
         GradBoxes gb;
         gb.full = gfull + 2 * ew;
@@ -623,9 +635,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                     for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
                     if (lane == 0 && active) rd[4 * BN + q] = lsum;
                 }
-                named_barrier_epi();   // (one per tile: `rd` is written again two tiles on, behind the next one)
+                named_barrier_epi<32 * C::WARPS>();   // (one per tile: `rd` is written again two tiles on, behind the next one)
                 const int tt = tile_ok ? threadIdx.x - 64 : BN;
-                for (int col = tt; col < BN; col += 32 * kEpiWarps)
+                for (int col = tt; col < BN; col += 32 * C::WARPS)
                     a.colsum[(int64_t)mt * a.N + n0 + col] =
                         rd[col] + rd[BN + col] + rd[2 * BN + col] + rd[3 * BN + col];
                 if (EPI == kEpiOutLoss && tile_ok && tt == 0)

@@ -964,7 +964,7 @@ cudaError_t launch_gemm(const CUtensorMap &ta, const CUtensorMap &tb, GemmArgs a
     const int units = (PAIR ? (m_tiles + 1) / 2 : m_tiles) * n_tiles * splits;
     const int most = num_sms_current() / (PAIR ? 2 : 1);
     return launch_step(gemm_kernel<BN, EPI, PAIR>, dim3((unsigned)((PAIR ? 2 : 1) * (units < most ? units : most))),
-                       dim3(kThreads), smem, PAIR ? 2 : 1, st, ta, tb, a);
+                       dim3(Cfg<BN, EPI, PAIR>::THREADS), smem, PAIR ? 2 : 1, st, ta, tb, a);
 }
 
 // Widest N tile (256, 128, 64 or 16) that divides N.
@@ -973,13 +973,17 @@ inline int pick_bn(int N) { return (N % 256 == 0) ? 256 : (N % 128 == 0) ? 128 :
 // CTA pairs take the N tiles that halve into whole boxes, where there are two
 // M-tiles to pair up and more than one k-block: with one the pair's coupling
 // costs more than its shared loads save (hidden layer, 65536 x 512 x 64: 34 us
-// on pairs, 27 on single CTAs; input gradient 39 and 32).
+// on pairs, 27 on single CTAs; input gradient 39 and 32).  The plain GEMM, held
+// by its stores where K is small, from K = 2048 on (single CTAs | pairs: 65536 x
+// 512 x 512 57 | 61 us, 8192 x 256 x 1024 12.6 | 13.4, x 2048 16.9 | 17.9, 65536
+// x 512 x 2048 120 | 108, 20000 x 1024 x 4096 133 | 113).
 template <int BN, int EPI>
 cudaError_t launch_gemm_pair(const CUtensorMap &ta, const CUtensorMap &tb, const GemmArgs &a, int m_tiles, int N,
                              int splits, cudaStream_t st)
 {
-    return m_tiles >= 2 && a.K > 64 ? launch_gemm<BN, EPI, true>(ta, tb, a, m_tiles, N / BN, splits, st)
-                        : launch_gemm<BN, EPI, false>(ta, tb, a, m_tiles, N / BN, splits, st);
+    constexpr int least = EPI == kEpiDw ? 2048 : 128;
+    return m_tiles >= 2 && a.K >= least ? launch_gemm<BN, EPI, true>(ta, tb, a, m_tiles, N / BN, splits, st)
+                                        : launch_gemm<BN, EPI, false>(ta, tb, a, m_tiles, N / BN, splits, st);
 }
 
 // Dispatch on the N tile width: 256 or 128 (hidden layers' widths are

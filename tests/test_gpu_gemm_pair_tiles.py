@@ -1,7 +1,8 @@
-"""GEMMs on CTA pairs (two or more M-tiles and K above 64) against single CTAs
-(128 rows at a time), bit for bit: pairs that take several tiles, so that the
-double-buffered accumulator and the stage ring come round, odd M-tile counts
-and ragged rows, every row compared; and K = 64, which stays on single CTAs."""
+"""GEMMs on CTA pairs (two or more M-tiles and K of 2048 and more) against
+single CTAs (128 rows at a time), bit for bit: pairs that take several tiles,
+so that the double-buffered accumulator and the stage ring come round, odd
+M-tile counts and ragged rows, every row compared; and smaller K, on single
+CTAs that take several tiles."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -10,7 +11,8 @@ pytestmark = pytest.mark.gpu
 # tiles of 128 or 256 columns; (20000, 1024, 320): 79 pair rows x 4 tiles on 76 pairs;
 # (40000, 128, 192): 157 pair rows, the last one's second M-tile missing (313 M-tiles)
 @pytest.mark.parametrize("M,N,K", [(129, 128, 128), (256, 256, 192), (20000, 1024, 320), (40000, 128, 192),
-                                   (19999, 512, 1024), (20000, 1024, 64)])
+                                   (19999, 512, 1024), (20000, 1024, 64), (129, 128, 2048), (256, 256, 2112),
+                                   (20000, 1024, 2112), (40000, 128, 2048), (19999, 512, 4096)])
 def test_every_row(prlib, cuda, M, N, K):
     import torch
     from paper_2312_04830_gb300 import binding
