@@ -4,17 +4,44 @@
 
 namespace prk {
 
-// A cell of the inversion's queue through the safeguarded iteration (from its
-// first evaluation when it has one), general form.
-static __device__ __noinline__ void newton_finish9(const NewtonArgs<double> &a, int64_t i, double T0, bool first,
-                                                   double h0, double cp0)
+// What a queued cell brings beside its start: nothing, its first evaluation,
+// or the FP32 cp at a warm root outside the fixed-point range.  (Evaluated where
+// it is found, such a root holds back its warp's other cells: 300000 cells, one
+// in six above 4096 K, 471 us, queued 372.)
+enum QueuedAs : unsigned char { kStartOnly = 0, kEvaluated = 1, kWarmRoot = 2 };
+
+// A cell of the inversion's queue, general form: one evaluation at a warm
+// root and the one-step acceptance, else the safeguarded iteration (from the
+// first evaluation when there is one).
+static __device__ __noinline__ void newton_finish9(const NewtonArgs<double> &a, const SpeciesRec<float> *sp32, int64_t i,
+                                                   double T0, int as, double h0, double cp0)
 {
     Comp<double, 9> c;
     double Tres = M<double>::nan(), cp_last;
     int it = 0, st = kBadInput;
-    if (load_comp<double, 9>(c, a.Y, a.ldY, i, a.N, a.sp))
-        st = newton_solve<double, double, 9, false>(c, __ldg(a.hstar + i), __ldg(a.p + i), T0, a.sp, a.kij, a.tmid_u,
-                                                    a.max_iter, a.rtol, 1e-6, Tres, it, cp_last, first, h0, cp0);
+    if (load_comp<double, 9>(c, a.Y, a.ldY, i, a.N, a.sp)) {
+        const double hs = __ldg(a.hstar + i), p = __ldg(a.p + i);
+        bool accepted = false;
+        if (as == kWarmRoot) {
+            FirstEval f = eval_h_first<double, double, 9, false>(c, T0, p, a.sp, a.kij, a.tmid_u);
+            if (f.status == kNoRoot) {
+                as = kStartOnly;
+            } else {
+                f.cp = cp0;
+                h0 = f.h;
+                const double dT = m64::div(hs - f.h, f.cp);
+                if (one_step_ok<9>(f, T0, dT, c.Wbar, sp32, (float)a.tmid_u)) {
+                    accepted = true;
+                    Tres = T0 + dT;
+                    st = kOk;
+                    it = 1;
+                }
+            }
+        }
+        if (!accepted)
+            st = newton_solve<double, double, 9, false>(c, hs, p, T0, a.sp, a.kij, a.tmid_u, a.max_iter, a.rtol, 1e-6,
+                                                        Tres, it, cp_last, as != kStartOnly, h0, cp0);
+    }
     a.Tout[i] = Tres;
     a.status[i] = st;
     if (a.iters) a.iters[i] = it;
@@ -69,7 +96,7 @@ __global__ void __launch_bounds__(kBlock) newton_warm_kernel(const __grid_consta
 __device__ __forceinline__ void newton_fix_cell(const NewtonArgs<double> &a, const Fix9 &t, int64_t i, double T,
                                                 float cp32, const SpeciesRec<float> *sp32, int *q_n,
                                                 int64_t *q_i, double *q_T, double *q_h, double *q_cp,
-                                                unsigned char *q_first, bool guess_ok)
+                                                unsigned char *q_as, bool guess_ok)
 {
     const double hs = __ldg(a.hstar + i), p = __ldg(a.p + i);
     double y[9];
@@ -83,17 +110,21 @@ __device__ __forceinline__ void newton_fix_cell(const NewtonArgs<double> &a, con
         if (a.iters) a.iters[i] = 0;
         return;
     }
-    bool first = false;
-    double h0 = 0.0, cp0 = 0.0;
+    int as = cp32 > 0.f ? kWarmRoot : kStartOnly;
+    double h0 = 0.0, cp0 = (double)cp32;
     if (ok == kFixOk && cp32 > 0.f && fix9_range(T)) {
         Thermo<double> th;
         fix9_thermo(t, c, T, p, th);
+        as = kStartOnly;
+        // the acceptance's table loads stay below the evaluation, whose registers
+        // they would take (2.1 M cells 698 us without this line, 642 with it)
+        asm volatile("" ::: "memory");
         if (th.status != kNoRoot) {
             FirstEval f;
             f.status = th.status;
             f.nroots = th.nroots;
             f.h = th.h;
-            f.cp = (double)cp32;
+            f.cp = cp0;
             f.cv_ig = (float)th.cv_ig_molar;
             const double dT = m64::div(hs - f.h, f.cp);
             if (one_step_ok<9>(f, T, dT, c.Wbar, sp32, (float)a.tmid_u)) {
@@ -102,9 +133,8 @@ __device__ __forceinline__ void newton_fix_cell(const NewtonArgs<double> &a, con
                 if (a.iters) a.iters[i] = 1;
                 return;
             }
-            first = true;
+            as = kEvaluated;
             h0 = f.h;
-            cp0 = f.cp;
         }
     }
     const int e = atomicAdd(q_n, 1);
@@ -112,7 +142,7 @@ __device__ __forceinline__ void newton_fix_cell(const NewtonArgs<double> &a, con
     q_T[e] = T;
     q_h[e] = h0;
     q_cp[e] = cp0;
-    q_first[e] = first ? 1 : 0;
+    q_as[e] = (unsigned char)as;
 }
 
 // SPLIT: T and cp from newton_warm_kernel; else the warm start runs here.
@@ -124,17 +154,17 @@ __global__ void __launch_bounds__(kBlock, 4) newton_fix_kernel(const __grid_cons
     __shared__ int q_n;
     __shared__ int64_t q_i[2 * kBlock];
     __shared__ double q_T[2 * kBlock], q_h[2 * kBlock], q_cp[2 * kBlock];
-    __shared__ unsigned char q_first[2 * kBlock];
+    __shared__ unsigned char q_as[2 * kBlock];
     if (threadIdx.x == 0) q_n = 0;
     stage<float, 9, false>(s32, a.sp32, a.pair32, a.kij32);   // ends with a barrier
-    auto finish = [&](int e) { newton_finish9(a, q_i[e], q_T[e], q_first[e] != 0, q_h[e], q_cp[e]); };
+    auto finish = [&](int e) { newton_finish9(a, s32.sp, q_i[e], q_T[e], q_as[e], q_h[e], q_cp[e]); };
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.n; base += stride) {
         const int64_t i = base + threadIdx.x;
         if (i < a.n) {
             if constexpr (SPLIT) {
                 const float cp32 = __int_as_float(a.status[i]);
-                newton_fix_cell(a, t, i, a.Tout[i], cp32, s32.sp, &q_n, q_i, q_T, q_h, q_cp, q_first, cp32 >= 0.f);
+                newton_fix_cell(a, t, i, a.Tout[i], cp32, s32.sp, &q_n, q_i, q_T, q_h, q_cp, q_as, cp32 >= 0.f);
             } else {
                 const double Tg = __ldg(a.Tg + i);
                 double y[9];
@@ -146,7 +176,7 @@ __global__ void __launch_bounds__(kBlock, 4) newton_fix_kernel(const __grid_cons
                 float cp32;
                 const double T = warm_start_fp32<9, false>(cf, fmin(fmax(Tg, kTLo), kTHi), __ldg(a.hstar + i),
                                                            __ldg(a.p + i), s32.sp, s32.kij, (float)a.tmid_u, wok, cp32);
-                newton_fix_cell(a, t, i, T, wok ? cp32 : 0.f, s32.sp, &q_n, q_i, q_T, q_h, q_cp, q_first, isfinite(Tg));
+                newton_fix_cell(a, t, i, T, wok ? cp32 : 0.f, s32.sp, &q_n, q_i, q_T, q_h, q_cp, q_as, isfinite(Tg));
             }
         }
         queue_round(&q_n, (int)threadIdx.x, (int)blockDim.x, finish);
