@@ -61,7 +61,7 @@ ALGO_FP64_FLOPS_PER_CELL = {"props_fp64": 1698.6035400390624}
 # / cells) of the same captures; a full launch moves this x its cells (the
 # forward surrogate: DRAM bytes per row of one resident-activation inference
 # launch over a 2 Mi-row chunk of the 128^3 field)
-TRAFFIC_BYTES_PER_CELL = {"props_fp64": 124.6, "newton_fp64": 226.4, "surrogate_bf16": 151.8}
+TRAFFIC_BYTES_PER_CELL = {"props_fp64": 124.6, "newton_fp64": 227.3, "surrogate_bf16": 151.8}
 # Instructions per cell the FP32 property kernel issues (ncu smsp__inst_executed.sum
 # x 32 / cells, one full launch on the 128^3 flame-vortex field): the kernel is
 # issue-bound, so its roofline is the issue rate, one warp instruction per

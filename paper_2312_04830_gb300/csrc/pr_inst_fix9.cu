@@ -203,8 +203,8 @@ void launch_newton_fix(const NewtonArgs<double> &a, const Fix9 &t, const void *h
                      !overlap(a.status, nb / 2, a.Y, yb) && !overlap(a.status, nb / 2, a.Tg, nb);
     // two launches for more cells than one wave of the single kernel holds:
     // up to there the second launch costs more than the smaller kernels gain
-    // (65536 cells, in one wave: 68 us against 71; 131072: 118 against 88;
-    // 2.1 M cells: 1216 against 692)
+    // (65536 cells, in one wave: 63 us against 65; 131072: 107 against 82;
+    // 2.1 M cells: 1176 against 641)
     if (a.n > (int64_t)occ[2] * sms * kBlock && own) {
         newton_warm_kernel<<<grid_for(a.n, occ[0], sms), kBlock, 0, st>>>(a, make_tab<float, 9, false>(htab32), t.warm);
         newton_fix_kernel<true><<<grid_for(a.n, occ[1], sms), kBlock, 0, st>>>(a, t);
